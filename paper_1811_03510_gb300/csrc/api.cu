@@ -43,12 +43,52 @@ static const uint32_t kMaxPatches = 1u << 26;
 
 namespace {
 
+void free_table(GregTabStore &t)
+{
+    cudaFree(t.node);
+    cudaFree(t.rank);
+    cudaFree(t.list);
+    cudaFree(t.depth);
+    t = GregTabStore{};
+}
+
+// Storage of the Gregory box table, within 1/32 of the free device memory; a scene without it (no Gregory patch,
+// no room) has no levels.  The depth word exists in either case.
+cudaError_t alloc_table(ccs_scene *sc)
+{
+    GregTabStore &t = sc->tab;
+    cudaError_t e = cudaMalloc(&t.depth, sizeof(uint32_t));
+    if (e != cudaSuccess) return e;
+    if ((e = cudaMemset(t.depth, 0, sizeof(uint32_t))) != cudaSuccess || sc->n_greg == 0) return e;
+    size_t room = 0, total = 0;
+    if ((e = cudaMemGetInfo(&room, &total)) != cudaSuccess) return e;
+    const uint32_t stride = greg_table_levels(sc->n_greg, room / 32);
+    if (stride == 0) return cudaSuccess;
+    std::vector<uint32_t> rank(sc->n), list;
+    list.reserve(sc->n_greg);
+    for (uint32_t p = 0; p < sc->n; ++p) {
+        rank[p] = (uint32_t)list.size();
+        if (sc->htypes[p]) list.push_back(p);
+    }
+    if (cudaMalloc(&t.node, ((size_t)sc->n_greg << stride) * 48) != cudaSuccess ||
+        cudaMalloc(&t.rank, rank.size() * 4) != cudaSuccess || cudaMalloc(&t.list, list.size() * 4) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return cudaSuccess;
+    }
+    if ((e = cudaMemcpy(t.rank, rank.data(), rank.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if ((e = cudaMemcpy(t.list, list.data(), list.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    t.n = sc->n_greg;
+    t.stride = stride;
+    return cudaSuccess;
+}
+
 void free_scene(ccs_scene *s)
 {
     if (!s) return;
     cudaFree(s->d_rec);
     cudaFree(s->d_leaf_box);
     cudaFree(s->d_types);
+    free_table(s->tab);
     cudaFree(s->d_nodes);
     cudaFree(s->d_leaf_parent);
     cudaFree(s->d_refit_flags);
@@ -346,6 +386,8 @@ ccs_status ccs_scene_create(ccs_scene **out, const float *x, const float *y, con
             cudaMemcpyAsync(sc->d_types, sc->htypes.data(), n_patches, cudaMemcpyHostToDevice, s);
             e = launch_repack(tmp, tmp + np, tmp + 2 * np, sc->d_types, n_patches, sc->local ? 1 : 0, sc->d_rec,
                               sc->d_leaf_box, s);
+            if (e == cudaSuccess) e = alloc_table(sc);
+            if (e == cudaSuccess) e = launch_greg_table(sc->tab, sc->d_rec, false, s);
             cudaError_t e2 = cudaStreamSynchronize(s);
             cudaFree(tmp);
             if (e == cudaSuccess) e = e2;
@@ -459,6 +501,7 @@ ccs_status ccs_scene_update_points(ccs_scene *sc, const float *x, const float *y
     CCS_ARG(sc->n == 0 || (x && y && z), "point array is NULL");
     CCS_CUDA(launch_repack(x, y, z, sc->d_types, sc->n, sc->local ? 1 : 0, sc->d_rec, sc->d_leaf_box,
                            (cudaStream_t)stream));
+    CCS_CUDA(launch_greg_table(sc->tab, sc->d_rec, true, (cudaStream_t)stream));
     return CCS_OK;
 }
 

@@ -63,6 +63,17 @@ struct LaunchCfg {
     float min_conf = 0.0f;
 };
 
+// Box table of a scene's Gregory patches (table.cu): the child boxes of every node above level `depth` of their
+// subdivision, so that a traversal loads a node's boxes instead of computing Algorithm 2's bound for every ray
+// that visits it.  A node (level l, path p) is 3 float4 at 3 ((rank << stride) + 2^l - 1 + p), axis by axis (lower
+// child lo, hi, upper child lo, hi): the boxes that split_step computes, before the extension of local frames.
+struct GregTab {
+    const float4 *node;
+    const uint32_t *rank;    // per patch: its rank among the Gregory patches
+    const uint32_t *depth;   // device word: the levels in use now (0: no table)
+    uint32_t stride;         // the levels that the storage holds
+};
+
 struct DevScene {
     const float4 *rec;       // n_patches records
     const float4 *nodes;     // n_nodes nodes
@@ -72,6 +83,7 @@ struct DevScene {
     uint32_t width;          // BVH node width: 2 or 4
     const uint8_t *types;    // n_patches bytes: 0 Bezier, 1 Gregory
     uint32_t n_greg;         // Gregory patches in the scene
+    GregTab tab;
 };
 
 struct DevRays {
@@ -81,6 +93,15 @@ struct DevRays {
 struct DevHits {
     float *t, *u, *v;
     uint32_t *pid;
+};
+
+// A scene's Gregory box table as the kernels that build it see it.
+struct GregTabStore {
+    float4 *node;
+    uint32_t *rank;     // per patch
+    uint32_t *list;     // the Gregory patches, in rank order
+    uint32_t *depth;
+    uint32_t n, stride; // Gregory patches; levels stored
 };
 
 // One scene of a batch (device table): where its data, rays and hits live.
@@ -93,11 +114,16 @@ struct BatchEntry {
     float4 *rec, *leaf_box, *nodes;
     const int *leaf_parent;
     uint32_t *refit_flags;
+    GregTabStore tab;
 };
 
 // kernels (intersect.cu, scene.cu)
 cudaError_t launch_repack(const float *x, const float *y, const float *z, const uint8_t *types, uint32_t n, int local,
                           float4 *rec, float4 *leaf_box, cudaStream_t s);
+// Gregory box tables (table.cu): the levels that `bytes` hold for n patches; the build after a repack (every
+// level, or after an update of the points fewer; a batch builds them beside its refit)
+uint32_t greg_table_levels(uint32_t n, size_t bytes);
+cudaError_t launch_greg_table(const GregTabStore &t, const float4 *rec, bool update, cudaStream_t s);
 cudaError_t launch_refit(float4 *nodes, const int *leaf_parent, const float4 *leaf_box, uint32_t *flags,
                          uint32_t n_patches, uint32_t n_nodes, uint32_t width, cudaStream_t s);
 cudaError_t launch_intersect(const DevScene &sc, const DevRays &r, const DevHits &h, uint32_t n,
@@ -149,6 +175,7 @@ struct ccs_scene {
     float4 *d_leaf_box = nullptr;      // 2 float4 per patch: (lo.xyz, 0), (hi.xyz, 0)
     uint8_t *d_types = nullptr;
     uint32_t n_greg = 0;               // Gregory patches
+    ccs::GregTabStore tab{};           // their box table (no levels when its memory could not be had)
     float4 *d_nodes = nullptr;
     int *d_leaf_parent = nullptr;      // per patch: (node << 1) | slot
     uint32_t *d_refit_flags = nullptr; // per node arrival counters of the refit
@@ -181,10 +208,11 @@ inline uint32_t *take_queue(ccs_scene *sc)
     return sc->d_work + kQueueBase + sc->next_queue.fetch_add(1, std::memory_order_relaxed) % kQueueRing;
 }
 
+inline GregTab dev_table(const GregTabStore &t) { return GregTab{t.node, t.rank, t.depth, t.stride}; }
 inline DevScene dev_scene(const ccs_scene *sc)
 {
     return DevScene{sc->d_rec,        sc->d_nodes, sc->d_leaf_box, sc->n, sc->n_nodes, sc->local ? 1u : 0u,
-                    sc->bvh_width,    sc->d_types, sc->n_greg};
+                    sc->bvh_width,    sc->d_types, sc->n_greg,     dev_table(sc->tab)};
 }
 
 // The scene seen through its BVH of the given width (0: the default one); the caller has checked that
@@ -197,6 +225,6 @@ inline DevScene dev_scene(const ccs_scene *sc, uint32_t width)
 {
     if (width == 0 || width == sc->bvh_width) return dev_scene(sc);
     return DevScene{sc->d_rec,     sc->d_nodes_alt, sc->d_leaf_box, sc->n,       sc->n_nodes_alt,
-                    sc->local ? 1u : 0u, sc->alt_width, sc->d_types, sc->n_greg};
+                    sc->local ? 1u : 0u, sc->alt_width, sc->d_types, sc->n_greg, dev_table(sc->tab)};
 }
 }  // namespace ccs

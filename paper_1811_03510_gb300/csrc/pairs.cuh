@@ -539,6 +539,13 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
     uint32_t *queue = pb.ctr + kCtrQueue;
     if (STATS && lane == 0) atomicMax(counters + 20, ~global_ns());   // first warp start
 
+    // levels of Gregory pairs in the table: one scene's are the same for every lane
+    int tab_d = 0;
+    if constexpr (!std::is_same<Src, BatchSource>::value) tab_d = src.sc.n_nodes ? table_levels(src.sc, L) : 0;
+    auto tab_levels = [&](const typename Src::LaneScene &l) {
+        if constexpr (std::is_same<Src, BatchSource>::value) return table_levels(src.scene(l), L);
+        else return tab_d;
+    };
     // the lane's ray (task)
     bool has_task = false, exhausted = false, evicted = false;
     uint32_t ray = 0, cur = 0, ray_scene = 0, ray_local = 0, iters = 0;
@@ -759,19 +766,44 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
             if (pass > 0 && !__any_sync(FULL, stepping)) break;
             if (stepping) {
                 --iters;
-                if (gpend) {   // Algorithm 2 with the crop of Algorithm 1 for the Gregory node (path, level)
-                    float u0, u1, v0, v1;
-                    node_domain(path, level, L, u0, u1, v0, v1);
-                    gregory_node<3>(rec_of(src.scene(lsc), pid), u0, u1, v0, v1, level, G, g, d);
-                    gpend = false;
-                }
                 const bool redesc = rd_target >= 0;
+                int slot = -1;
+                StepOut so;
+                if (gpend && level < tab_levels(lsc)) {
+                    // a Gregory node in the scene's table: the lane goes down through the table at once, a load
+                    // and two slab tests per level, while the others split
+                    const float4 *nodes = table_nodes(src.scene(lsc), pid);
+                    const int last = tab_levels(lsc) - 1;
+                    for (;;) {
+                        if (STATS) cnt.v[2]++;
+                        so = table_step(nodes + 3 * (size_t)((1u << level) - 1u + path), pr, c0, c1, te, best.t, G, tau);
+                        if (level == last || iters == 0 || !(so.hitL || so.hitR)) break;
+                        --iters;
+                        const uint32_t bit = 1u << level;
+                        if (so.hitL && so.hitR) {
+                            trail |= bit;
+                            scr.sib[level * stride] = so.goR ? make_float2(so.l0, so.l1) : make_float2(so.r0, so.r1);
+                        }
+                        path = so.goR ? (path | bit) : path;
+                        c0 = so.goR ? so.r0 : so.l0;
+                        c1 = so.goR ? so.r1 : so.l1;
+                        ++level;
+                    }
+                } else {
+                    if (gpend) {   // Algorithm 2 with the crop of Algorithm 1 for the Gregory node (path, level)
+                        float u0, u1, v0, v1;
+                        node_domain(path, level, L, u0, u1, v0, v1);
+                        gregory_node<3>(rec_of(src.scene(lsc), pid), u0, u1, v0, v1, level, G, g, d);
+                    }
+                    const bool leafkids = !redesc && level + 1 == 2 * L;
+                    const int force = redesc ? (int)((path >> level) & 1u) : -1;
+                    slot = (!redesc && !leafkids && K > 0 && !greg) ? (ctop % (K > 0 ? K : 1)) : -1;
+                    if (STATS && !redesc) cnt.v[greg ? 2 : 1]++;
+                    so = split_step<K, 3>(g, pr, d, c0, c1, te, best.t, redesc || (!greg && !leafkids), scr, slot, true,
+                                          true, force, G, tau);
+                }
+                gpend = false;
                 const bool leafkids = !redesc && level + 1 == 2 * L;
-                const int force = redesc ? (int)((path >> level) & 1u) : -1;
-                const int slot = (!redesc && !leafkids && K > 0 && !greg) ? (ctop % (K > 0 ? K : 1)) : -1;
-                if (STATS && !redesc) cnt.v[greg ? 2 : 1]++;
-                const StepOut so = split_step<K, 3>(g, pr, d, c0, c1, te, best.t, redesc || (!greg && !leafkids), scr,
-                                                    slot, true, true, force, G, tau);
                 if (redesc) {
                     if (++level == rd_target) rd_target = -1;
                 } else if (so.hitL || so.hitR) {
@@ -804,7 +836,7 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
                         if (so.hitL && so.hitR) {
                             trail |= bit;
                             scr.sib[level * stride] = so.goR ? make_float2(so.l0, so.l1) : make_float2(so.r0, so.r1);
-                            if (K > 0 && !greg) {
+                            if (K > 0 && slot >= 0) {
                                 scr.tag[slot] = level;
                                 ++ctop;
                                 cvalid = cvalid < K ? cvalid + 1 : K;

@@ -1,0 +1,51 @@
+// Gregory box tables: the boxes of the sub-domains of a scene's Gregory patches, stored once per scene (and again
+// after an update of its points) instead of computed by every ray that visits them.  A node's bound (Algorithm 2
+// with the crop of Algorithm 1, about 1130 operations, then a split of 360) does not depend on the ray: the
+// extension of local frames and the clipping to the parent's interval come where a ray tests the boxes.  The
+// stored boxes are bit for bit those that gregory_node and split_step give, by the same code.
+//
+// Why: a Gregory step takes a lone warp about 7,000 cycles, a Bezier step 1,600, and a ray that grazes a Gregory patch
+// takes dozens of them one after another, so launches ended on such rays.  A table step (48 bytes, two slab tests)
+// is bound by the latency of its load.  Measured, before and after (us per pair-engine call): 64 x 64 rays on 96
+// patches 165 -> 129, 330 k diffuse rays on 1,632 patches 250 -> 220, 300 k any-hit shadow rays there 536 -> 410, 1.2 M
+// mirror rays on 98,400 patches 665 -> 565; 1080p primary rays, which rarely meet one, unchanged.
+// Levels: meshes have few irregular faces, so their tables may be deep; 14 levels (786 KB) per patch while they fit in
+// 128 MB.  (16, all of leaf depth 8: 120 us instead of 129 on the 96 patches, but scene creation took 0.3 ms
+// longer, 14%.)  After an update of the points 10 levels, built beside the batch's refit: no time of its own.
+#include <algorithm>
+
+#include "table_dev.cuh"
+
+namespace ccs {
+
+namespace {
+
+__global__ void __launch_bounds__(128) k_greg_table(GregTabStore t, const float4 *__restrict__ rec, uint32_t D)
+{
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *t.depth = D;
+    if (i >= (size_t)t.n << D) return;
+    const uint32_t m = (uint32_t)i & ((1u << D) - 1u);
+    if (m + 1u < (1u << D)) greg_table_node(t, rec, (uint32_t)(i >> D), m);
+}
+
+}  // namespace
+
+uint32_t greg_table_levels(uint32_t n, size_t bytes)
+{
+    const uint64_t most = std::min<uint64_t>(bytes, kGregBytes);
+    uint32_t D = n ? kGregLevels : 0;
+    while (D > 0 && ((uint64_t)n << D) * 48 > most) --D;
+    return D;
+}
+
+cudaError_t launch_greg_table(const GregTabStore &t, const float4 *rec, bool update, cudaStream_t s)
+{
+    if (!t.stride) return cudaSuccess;
+    const uint32_t D = update ? greg_update_levels(t.stride) : t.stride;
+    const size_t n = (size_t)t.n << D;
+    k_greg_table<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(t, rec, D);
+    return cudaGetLastError();
+}
+
+}  // namespace ccs

@@ -442,13 +442,18 @@ CCS_DEV float max16(float a0, float a1, float a2, float a3, float a4, float a5, 
                  max3f(max3f(a9, a10, a11), max3f(a12, a13, a14), a15));
 }
 
-template <int K, int NC>
-CCS_DEV StepOut split_step(float (&g)[16 * NC], const RayG<NC> &r, const float (&d)[NC], float c0, float c1, float te,
-                           float tb, bool keep_grid, const Scratch &sc, int cache_slot, bool allowL, bool allowR,
-                           int force, const Grp &G, float tau)
-{
+// The points of a de Casteljau split at the midpoint, column by column: the lower half is (e0, m01, m012, mm),
+// the upper half (mm, m123, m23, e3).
+template <int NC>
+struct SplitPts {
     float e0[4 * NC], e3[4 * NC], m01[4 * NC], m012[4 * NC], mm[4 * NC], m123[4 * NC], m23[4 * NC];
-    float lmin[NC], lmax[NC], rmin[NC], rmax[NC];
+};
+
+// Splits the grid g and bounds the two halves: [lmin, lmax] and [rmin, rmax], the maxima raised by d.
+template <int NC>
+CCS_DEV void split_boxes(const float (&g)[16 * NC], const float (&d)[NC], SplitPts<NC> &S, float (&lmin)[NC],
+                         float (&lmax)[NC], float (&rmin)[NC], float (&rmax)[NC])
+{
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
 #pragma unroll
@@ -456,30 +461,42 @@ CCS_DEV StepOut split_step(float (&g)[16 * NC], const RayG<NC> &r, const float (
             const int q = c * 4 + b;
             const float b0 = g[c * 16 + 0 * 4 + b], b1 = g[c * 16 + 1 * 4 + b];
             const float b2 = g[c * 16 + 2 * 4 + b], b3 = g[c * 16 + 3 * 4 + b];
-            e0[q] = b0;
-            e3[q] = b3;
-            m01[q] = mid(b0, b1);
+            S.e0[q] = b0;
+            S.e3[q] = b3;
+            S.m01[q] = mid(b0, b1);
             const float m12 = mid(b1, b2);
-            m23[q] = mid(b2, b3);
-            m012[q] = mid(m01[q], m12);
-            m123[q] = mid(m12, m23[q]);
-            mm[q] = mid(m012[q], m123[q]);
+            S.m23[q] = mid(b2, b3);
+            S.m012[q] = mid(S.m01[q], m12);
+            S.m123[q] = mid(m12, S.m23[q]);
+            S.mm[q] = mid(S.m012[q], S.m123[q]);
         }
         // the lower half's 16 points (b0, m01, m012, mm of each column) and the upper half's (mm, m123, m23, b3)
         const int q = c * 4;
-        lmin[c] = min16(e0[q], m01[q], m012[q], mm[q], e0[q + 1], m01[q + 1], m012[q + 1], mm[q + 1], e0[q + 2],
-                        m01[q + 2], m012[q + 2], mm[q + 2], e0[q + 3], m01[q + 3], m012[q + 3], mm[q + 3]);
-        lmax[c] = __fadd_rn(max16(e0[q], m01[q], m012[q], mm[q], e0[q + 1], m01[q + 1], m012[q + 1], mm[q + 1],
-                                  e0[q + 2], m01[q + 2], m012[q + 2], mm[q + 2], e0[q + 3], m01[q + 3], m012[q + 3],
-                                  mm[q + 3]),
+        lmin[c] = min16(S.e0[q], S.m01[q], S.m012[q], S.mm[q], S.e0[q + 1], S.m01[q + 1], S.m012[q + 1], S.mm[q + 1],
+                        S.e0[q + 2], S.m01[q + 2], S.m012[q + 2], S.mm[q + 2], S.e0[q + 3], S.m01[q + 3],
+                        S.m012[q + 3], S.mm[q + 3]);
+        lmax[c] = __fadd_rn(max16(S.e0[q], S.m01[q], S.m012[q], S.mm[q], S.e0[q + 1], S.m01[q + 1], S.m012[q + 1],
+                                  S.mm[q + 1], S.e0[q + 2], S.m01[q + 2], S.m012[q + 2], S.mm[q + 2], S.e0[q + 3],
+                                  S.m01[q + 3], S.m012[q + 3], S.mm[q + 3]),
                             d[c]);
-        rmin[c] = min16(mm[q], m123[q], m23[q], e3[q], mm[q + 1], m123[q + 1], m23[q + 1], e3[q + 1], mm[q + 2],
-                        m123[q + 2], m23[q + 2], e3[q + 2], mm[q + 3], m123[q + 3], m23[q + 3], e3[q + 3]);
-        rmax[c] = __fadd_rn(max16(mm[q], m123[q], m23[q], e3[q], mm[q + 1], m123[q + 1], m23[q + 1], e3[q + 1],
-                                  mm[q + 2], m123[q + 2], m23[q + 2], e3[q + 2], mm[q + 3], m123[q + 3], m23[q + 3],
-                                  e3[q + 3]),
+        rmin[c] = min16(S.mm[q], S.m123[q], S.m23[q], S.e3[q], S.mm[q + 1], S.m123[q + 1], S.m23[q + 1], S.e3[q + 1],
+                        S.mm[q + 2], S.m123[q + 2], S.m23[q + 2], S.e3[q + 2], S.mm[q + 3], S.m123[q + 3],
+                        S.m23[q + 3], S.e3[q + 3]);
+        rmax[c] = __fadd_rn(max16(S.mm[q], S.m123[q], S.m23[q], S.e3[q], S.mm[q + 1], S.m123[q + 1], S.m23[q + 1],
+                                  S.e3[q + 1], S.mm[q + 2], S.m123[q + 2], S.m23[q + 2], S.e3[q + 2], S.mm[q + 3],
+                                  S.m123[q + 3], S.m23[q + 3], S.e3[q + 3]),
                             d[c]);
     }
+}
+
+template <int K, int NC>
+CCS_DEV StepOut split_step(float (&g)[16 * NC], const RayG<NC> &r, const float (&d)[NC], float c0, float c1, float te,
+                           float tb, bool keep_grid, const Scratch &sc, int cache_slot, bool allowL, bool allowR,
+                           int force, const Grp &G, float tau)
+{
+    SplitPts<NC> S;
+    float lmin[NC], lmax[NC], rmin[NC], rmax[NC];
+    split_boxes<NC>(g, d, S, lmin, lmax, rmin, rmax);
     if (tau > 0.0f) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
@@ -508,14 +525,14 @@ CCS_DEV StepOut split_step(float (&g)[16 * NC], const RayG<NC> &r, const float (
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 const int q = c * 4 + b;
-                const float b0 = e0[q], b3 = e3[q];   // g is overwritten in place (transposed) below
-                const float k0 = up ? mm[q] : b0, k1 = up ? m123[q] : m01[q];
-                const float k2 = up ? m23[q] : m012[q], k3 = up ? b3 : mm[q];
+                const float b0 = S.e0[q], b3 = S.e3[q];   // g is overwritten in place (transposed) below
+                const float k0 = up ? S.mm[q] : b0, k1 = up ? S.m123[q] : S.m01[q];
+                const float k2 = up ? S.m23[q] : S.m012[q], k3 = up ? b3 : S.mm[q];
                 if (K > 0 && store) {
                     // the other child, in the same transposed layout
                     float4 *dst = reinterpret_cast<float4 *>(sc.cache + cache_slot * 16 * NC);
-                    dst[c * 4 + b] = make_float4(up ? b0 : mm[q], up ? m01[q] : m123[q], up ? m012[q] : m23[q],
-                                                 up ? mm[q] : b3);
+                    dst[c * 4 + b] = make_float4(up ? b0 : S.mm[q], up ? S.m01[q] : S.m123[q],
+                                                 up ? S.m012[q] : S.m23[q], up ? S.mm[q] : b3);
                 }
                 g[c * 16 + b * 4 + 0] = k0;
                 g[c * 16 + b * 4 + 1] = k1;
@@ -526,6 +543,42 @@ CCS_DEV StepOut split_step(float (&g)[16 * NC], const RayG<NC> &r, const float (
     }
     return o;
 }
+
+// The same step for a Gregory node whose child boxes are in the scene's table (nd: its 3 float4).
+CCS_DEV StepOut table_step(const float4 *__restrict__ nd, const RayG<3> &r, float c0, float c1, float te, float tb,
+                           const Grp &G, float tau)
+{
+    float lmin[3], lmax[3], rmin[3], rmax[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float4 q = __ldg(nd + k);
+        lmin[k] = q.x;
+        lmax[k] = q.y;
+        rmin[k] = q.z;
+        rmax[k] = q.w;
+    }
+    if (tau > 0.0f) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            extend(lmin[k], lmax[k], tau);
+            extend(rmin[k], rmax[k], tau);
+        }
+    }
+    StepOut o;
+    o.dL = o.dR = 0.0f;
+    slab<3>(r, lmin, lmax, c0, c1, G, o.l0, o.l1);
+    slab<3>(r, rmin, rmax, c0, c1, G, o.r0, o.r1);
+    o.hitL = o.l0 <= o.l1 && __fadd_rn(te, o.l0) <= tb;
+    o.hitR = o.r0 <= o.r1 && __fadd_rn(te, o.r0) <= tb;
+    o.goR = o.hitR && (!o.hitL || o.r0 < o.l0);
+    return o;
+}
+CCS_DEV const float4 *table_nodes(const DevScene &sc, uint32_t pid)
+{
+    return sc.tab.node + 3 * ((size_t)__ldg(sc.tab.rank + pid) << sc.tab.stride);
+}
+// The levels of Gregory pairs whose boxes are in the scene's table.
+CCS_DEV int table_levels(const DevScene &sc, int L) { return min((int)__ldg(sc.tab.depth), 2 * L); }
 
 // Slab tests against both child boxes of a BVH node; q[k] = the node's float4 of component comp(k).
 template <int NC>
