@@ -248,8 +248,8 @@ __global__ void __launch_bounds__(128, MINB) k_intersect(Src src, int L, uint32_
                                   k + 1 < kFeat ? f[k + 1] : 0.0f);
                 }
                 __syncwarp();
-                if (need & 0x0000ffffu) mlp_round(*mw, *mt, 0, lane, nullptr, 0u);
-                if (need & 0xffff0000u) mlp_round(*mw, *mt, 1, lane, nullptr, 0u);
+                if (need & 0x0000ffffu) mlp_round(*mw, *mt, 0, lane);
+                if (need & 0xffff0000u) mlp_round(*mw, *mt, 1, lane);
                 if (mine) {
                     if (mt->pmax[lane] >= min_conf) {
                         s.phase = kPhaseDirected;

@@ -84,10 +84,36 @@ __device__ __forceinline__ void mlp_layer(const __nv_bfloat16 *in, int in_stride
     }
 }
 
+// Argmax (ties: the lowest) and softmax normaliser, sum of exp(v - max), of row h (0 or 1) of a quad's result tile over
+// its 64 columns.
+__device__ __forceinline__ void quad_argmax(const float (&acc)[8][4], int h, int t, float &best, int &bidx, float &sum)
+{
+    best = -__int_as_float(0x7f800000);
+    bidx = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float v = acc[j][2 * h + e];
+            const int c = 8 * j + 2 * t + e;
+            if (v > best) { best = v; bidx = c; }
+        }
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
+        if (ov > best || (ov == best && oi < bidx)) { best = ov; bidx = oi; }
+    }
+    sum = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum += __expf(acc[j][2 * h] - best) + __expf(acc[j][2 * h + 1] - best);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+}
+
 // Forward pass of rows [16*r, 16*r+16) of the warp's x tile; writes argmax cell and max softmax
-// probability per row into the tiles (ties: lowest cell), and optionally the logits (row stride 64).
-__device__ __forceinline__ void mlp_round(const MlpWeights &W, MlpWarpTiles &T, int r, int lane, float *logits_out,
-                                          uint32_t rows_valid)
+// probability per row into the tiles (ties: lowest cell).
+__device__ __forceinline__ void mlp_round(const MlpWeights &W, MlpWarpTiles &T, int r, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
     float acc[8][4];
@@ -99,38 +125,13 @@ __device__ __forceinline__ void mlp_round(const MlpWeights &W, MlpWarpTiles &T, 
     // argmax and softmax normaliser of rows g and g + 8 over the quad's 64 columns
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        float best = -__int_as_float(0x7f800000);
-        int bidx = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const float v = acc[j][2 * h + e];
-                const int c = 8 * j + 2 * t + e;
-                if (v > best) { best = v; bidx = c; }
-            }
-#pragma unroll
-        for (int o = 1; o <= 2; o <<= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-            if (ov > best || (ov == best && oi < bidx)) { best = ov; bidx = oi; }
-        }
-        float sum = 0.0f;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) sum += __expf(acc[j][2 * h] - best) + __expf(acc[j][2 * h + 1] - best);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+        float best, sum;
+        int bidx;
+        quad_argmax(acc, h, t, best, bidx, sum);
         const int row = 16 * r + g + 8 * h;
         if (t == 0) {
             T.cell[row] = (uint8_t)bidx;
             T.pmax[row] = 1.0f / sum;
-        }
-        if (logits_out && ((rows_valid >> row) & 1u)) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                logits_out[row * kCells + 8 * j + 2 * t] = acc[j][2 * h];
-                logits_out[row * kCells + 8 * j + 2 * t + 1] = acc[j][2 * h + 1];
-            }
         }
     }
     __syncwarp();

@@ -1,5 +1,5 @@
-"""The proposal network's gradient kernel at the edges of its tiles (32 rows; blocks take several tiles from 304 tiles
-on, 9,728 rows), with buffers that are not aligned for wide accesses."""
+"""The proposal network's gradient and inference kernels at the edges of their tiles (32 rows; the gradient's blocks
+take several tiles from 304 tiles on, 9,728 rows), with buffers that are not aligned for wide accesses."""
 import numpy as np
 import pytest
 
@@ -59,3 +59,28 @@ def test_gradient_at_the_edges_of_its_tiles(B):
     assert torch.equal(*out)
     for h in (p, q):
         ccs.ccs_proposal_destroy(h)
+
+
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 31, 32, 33, 129, 58400])
+def test_inference_rows_do_not_depend_on_their_tile(n):
+    p = ccs.ccs_proposal_create(seed=5)
+    m = 1 << 16
+    X = torch.randn(m, 24, device="cuda", generator=torch.Generator(device="cuda").manual_seed(n))
+    ref = [torch.empty(m, 64, device="cuda"), torch.empty(m, dtype=torch.uint8, device="cuda"), torch.empty(m, device="cuda")]
+    ccs.ccs_proposal_infer(p, X, m, *ref)
+    a = 7   # rows 7 .. 7 + n, in buffers that start at odd multiples of their element
+    Y = shifted((n, 24), torch.float32, 1)
+    Y.copy_(X[a:a + n])
+    out = [shifted((n, 64), torch.float32, 1), shifted((n,), torch.uint8, 1), shifted((n,), torch.float32, 1)]
+    ccs.ccs_proposal_infer(p, Y, n, *out)
+    torch.cuda.synchronize()
+    for got, want in zip(out, ref):
+        assert torch.equal(got, want[a:a + n])
+    # each result alone
+    for k in range(3):
+        one = [None, None, None]
+        one[k] = torch.empty_like(out[k])
+        ccs.ccs_proposal_infer(p, Y, n, *one)
+        torch.cuda.synchronize()
+        assert torch.equal(one[k], out[k])
+    ccs.ccs_proposal_destroy(p)
