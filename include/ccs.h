@@ -96,7 +96,14 @@ typedef struct {
                                  entry distance is a leaf, reported with u, v at its domain's centre and
                                  the cell index of its lowest leaf cell.  Changes the answer (it is a
                                  method parameter, not a launch option); one lane per ray.  [0] */
-    uint32_t flags;           /* CCS_TRACE_* bits */
+    uint32_t flags;           /* CCS_TRACE_* bits.  With none, and with block_threads, blocks_per_sm, chunk,
+                                 bvh_burst, min_blocks, vote, iter_cap and pixel_spread left 0 and
+                                 lanes_per_ray 0 or 1, the library picks the engine: ccs_intersect,
+                                 ccs_intersect_host, ccs_intersect_host_batches and ccs_occluded then run
+                                 the pair engine (CCS_TRACE_PAIRS, with the 1-slot cache for
+                                 CCS_CACHE_DEFAULT) for up to 2^23 rays (with local frames, from 2^14 rays
+                                 on) outside stream capture while its scratch can be had, and the
+                                 ray-persistent kernel otherwise */
     uint64_t *counters;       /* optional device array of CCS_NUM_COUNTERS uint64 (CCS_TRACE_COUNT) */
     uint32_t image_width;     /* the rays are an image of this width, ray y * width + x (the last row may
                                  be partial).  CCS_TRACE_ORDER: ordered in tiles of 8 x 8 pixels with

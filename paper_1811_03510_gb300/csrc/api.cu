@@ -127,6 +127,10 @@ ccs_status ccs::fill_launch_cfg(const ccs_trace_opts *o, LaunchCfg &c)
     c.host_chunk = o ? o->host_chunk : 0;
     c.bvh_width = o ? o->bvh_width : 0;
     c.counters = o ? reinterpret_cast<unsigned long long *>(o->counters) : nullptr;
+    // no flag and no option that only the ray-persistent kernel has
+    c.auto_engine = !o || (o->flags == 0 && !o->block_threads && !o->blocks_per_sm && !o->chunk && !o->bvh_burst &&
+                           !o->min_blocks && !o->vote && o->lanes_per_ray <= 1 && !o->iter_cap && o->pixel_spread == 0.0f);
+    c.auto_cache = !o || o->cache_slots == CCS_CACHE_DEFAULT;
     CCS_ARG(c.leaf_depth >= 1 && c.leaf_depth <= (uint32_t)kMaxLeafDepth, "leaf_depth must be in 1..15");
     CCS_ARG(c.block_threads % 32 == 0 && c.block_threads >= 32 && c.block_threads <= 128,
             "block_threads must be a multiple of 32 in 32..128");
@@ -534,6 +538,7 @@ ccs_status ccs_intersect(const ccs_scene *sc, const ccs_rays *rays, uint32_t n, 
     if ((st = fill_launch_cfg(opts, cfg)) != CCS_OK) return st;
     CCS_ARG(has_width(sc, cfg.bvh_width), "the scene has no BVH of the width opts->bvh_width asks for");
     if (cfg.pixel_spread > 0.0f) cfg.mode = 4;   // screen-space termination (one lane per ray)
+    choose_engine(cfg, sc->local, n, (cudaStream_t)stream);
     DevScene ds = dev_scene(sc, cfg.bvh_width);
     DevRays dr{rays->ox, rays->oy, rays->oz, rays->dx, rays->dy, rays->dz, rays->tmin, rays->tmax};
     DevHits dh{hits->t, hits->u, hits->v, hits->patch_id};
@@ -657,6 +662,7 @@ ccs_status ccs_intersect_host(ccs_scene *sc, const ccs_rays *hr, uint32_t n, ccs
             return CCS_OK;
         }
     }
+    choose_engine(cfg, sc->local, n, s);
     const HostBatch one{hr, n, hh, cfg};
     return host_pipeline(sc, &one, 1, s);
 }
@@ -679,6 +685,7 @@ ccs_status ccs_intersect_host_batches(ccs_scene *sc, uint32_t n_batches, const c
         if ((st = fill_launch_cfg(opts ? opts[j] : nullptr, cfg)) != CCS_OK) return st;
         CCS_ARG(has_width(sc, cfg.bvh_width), "the scene has no BVH of the width opts->bvh_width asks for");
         if (cfg.pixel_spread > 0.0f) cfg.mode = 4;
+        choose_engine(cfg, sc->local, n[j], (cudaStream_t)stream);
         bt[j] = HostBatch{&hr[j], n[j], &hh[j], cfg};
     }
     return host_pipeline(sc, bt.data(), n_batches, (cudaStream_t)stream);
@@ -743,6 +750,7 @@ ccs_status ccs_occluded(const ccs_scene *sc, const ccs_rays *rays, uint32_t n, u
     CCS_ARG(has_width(sc, cfg.bvh_width), "the scene has no BVH of the width opts->bvh_width asks for");
     cfg.mode = 3;
     cfg.mc.occluded = occluded;
+    choose_engine(cfg, sc->local, n, (cudaStream_t)stream);
     DevScene ds = dev_scene(sc, cfg.bvh_width);
     DevRays dr{rays->ox, rays->oy, rays->oz, rays->dx, rays->dy, rays->dz, rays->tmin, rays->tmax};
     DevHits dh{nullptr, nullptr, nullptr, nullptr};

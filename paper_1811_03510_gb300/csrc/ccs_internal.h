@@ -57,6 +57,8 @@ struct LaunchCfg {
         lanes_per_ray, iter_cap, flags, image_width, host_chunk, bvh_width;
     float pixel_spread;
     unsigned long long *counters;
+    bool auto_engine = false;             // the options leave the engine to the library (choose_engine)
+    bool auto_cache = false;              // and the sibling cache
     int mode = 0;                         // 0 plain, 1 trace export, 2 learned proposal, 3 any hit, 4 screen-space
     ModeCtx mc{};
     const MlpWeights *mlp = nullptr;
@@ -140,6 +142,8 @@ cudaError_t launch_intersect_batch(const BatchEntry *entries, const uint32_t *ra
 // pair engine (pairs.cu): whether a launch with these options runs it, its scratch for n rays, and the
 // launches (single scene: scratch from the library's stream-ordered pool; batch: the caller's scratch)
 bool use_pairs(const LaunchCfg &cfg);
+// the engine of a launch of n rays on stream s whose options leave it open
+void choose_engine(LaunchCfg &cfg, bool local, uint32_t n, cudaStream_t s);
 size_t pairs_scratch_bytes(uint32_t n);
 // scratch of one launch from the library's stream-ordered memory pool of the current device (pairs.cu):
 // allocated and freed in the order of `s`; freed memory stays in the pool for reuse

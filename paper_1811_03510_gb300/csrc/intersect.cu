@@ -18,7 +18,11 @@ extern template cudaError_t launch_batch_w<4>(const BatchEntry *, const uint32_t
 cudaError_t launch_intersect(const DevScene &sc, const DevRays &r, const DevHits &h, uint32_t n, const LaunchCfg &cfg,
                              uint32_t *queue, uint32_t *status, int num_sms, cudaStream_t s, const uint32_t *perm)
 {
-    if (use_pairs(cfg)) return launch_pairs_single(sc, r, h, n, cfg, status, num_sms, s);
+    if (use_pairs(cfg)) {
+        const cudaError_t e = launch_pairs_single(sc, r, h, n, cfg, status, num_sms, s);
+        if (!(e == cudaErrorMemoryAllocation && cfg.auto_engine)) return e;
+        (void)cudaGetLastError();   // no room for its scratch: the ray-persistent kernel needs none
+    }
     return sc.width == 4 ? launch_single_w<4>(sc, r, h, n, cfg, queue, status, num_sms, s, perm)
                          : launch_single_w<2>(sc, r, h, n, cfg, queue, status, num_sms, s, perm);
 }

@@ -14,6 +14,29 @@ bool use_pairs(const LaunchCfg &cfg)
            cfg.lanes_per_ray == 1;
 }
 
+// The engine of a launch that leaves it open, by both engines' times over images and their bounce rays (96 to 98,304
+// patches, 16 x 16 to 1283 x 717 pixels; ray-persistent / pair engine).  World-axis boxes: the pair engine at every
+// size (1283 x 717 image 1484 / 676 us on 1,536 patches, 16 x 16 225 / 170; bounce rays 1.1 to 3.3 times faster, but
+// 0.93 times for 153,000 rays on 24,576 patches or more).  Local frames: from 2^14 rays on (1283 x 717 image 553 / 242
+// us, 256 x 144 1.04 to 1.55 times faster); below, its three launches and its tail cost what it saves (64 x 64 0.87 to
+// 1.11 times, 6,144 bounce rays 0.75 to 1.28).  With the 1-slot sibling cache, its fastest on images.
+// Not above 2^23 rays (an 8.3 M pixel image fits), whose scratch of 1.6 GB the library's pool would keep, and not while
+// the stream is captured, where the ray-persistent kernel needs no allocation; that kernel also takes the launch when
+// the scratch cannot be had (launch_intersect).
+void choose_engine(LaunchCfg &cfg, bool local, uint32_t n, cudaStream_t s)
+{
+    constexpr uint32_t kLeastLocal = 1u << 14, kMostRays = 1u << 23;
+    if (!cfg.auto_engine || n > kMostRays || (local && n < kLeastLocal)) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return;
+    cfg.flags |= CCS_TRACE_PAIRS;
+    if (cfg.auto_cache) cfg.cache_slots = 1;
+}
+
 size_t pairs_scratch_bytes(uint32_t n) { return pair_scratch_bytes(n); }
 
 namespace {

@@ -48,7 +48,7 @@ def test_table_hits_equal_the_ray_kernel(n, depth, local):
     r = sg.random_rays(6001, seed=90 + depth, target=1.05)
     rays = ccs.rays_to_device(r.soa())
     sc = ccs.Scene(P, types, local=local)
-    ref = trace(sc, rays, r.n, leaf_depth=depth)
+    ref = trace(sc, rays, r.n, leaf_depth=depth, chunk=32)   # an option that only that kernel has
     assert (ref["pid"] != 0xFFFFFFFF).sum() > 1000
     for K in (0, 1):
         same(trace(sc, rays, r.n, leaf_depth=depth, pairs=True, cache_slots=K), ref, K)
@@ -70,7 +70,7 @@ def test_table_follows_updates_of_the_points():
     ccs.ccs_bvh_refit(sc.handle)
     got = trace(sc, rays, r.n, pairs=True)
     assert (got["t"] != before["t"]).sum() > 1000
-    same(got, trace(sc, rays, r.n), "updated")
+    same(got, trace(sc, rays, r.n, chunk=32), "updated")
     sc.close()
     # the same through a batch of two scenes, one of them without a Gregory patch and one with new points
     flat = ccs.Scene(s.P, np.zeros_like(s.types), local=True)
@@ -82,7 +82,7 @@ def test_table_follows_updates_of_the_points():
     ccs.ccs_batch_run(b, stages, ccs.make_opts(pairs=True))
     assert ccs.ccs_batch_sync_status(b) == ccs.CCS_OK
     same(ccs.hits_to_numpy(hits[1]), got, "batch")
-    same(ccs.hits_to_numpy(hits[0]), trace(flat, rays, r.n), "batch, no table")
+    same(ccs.hits_to_numpy(hits[0]), trace(flat, rays, r.n, chunk=32), "batch, no table")
     ccs.ccs_batch_destroy(b)
     flat.close()
     sc.close()
