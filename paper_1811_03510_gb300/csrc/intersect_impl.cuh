@@ -40,6 +40,15 @@ struct SingleSource {
     CCS_DEV const DevHits &hits_of(uint32_t) const { return hits; }
 };
 
+// The same without a permutation (the pair engine has its own order).
+struct DirectSource : SingleSource {
+    CCS_DEV void locate(uint32_t i, LaneScene &, uint32_t &scene, uint32_t &local) const
+    {
+        scene = 0;
+        local = i;
+    }
+};
+
 // Rays of many scenes, concatenated in scene order (ray_prefix[s] = first global index of scene s).
 struct BatchSource {
     const BatchEntry *entries;

@@ -114,7 +114,7 @@ cudaError_t launch_pairs_single(const DevScene &sc, const DevRays &r, const DevH
     cudaError_t e = pool_alloc(&base, pair_scratch_bytes(n), s);
     if (e != cudaSuccess) return e;
     const PairBufs pb = pair_bufs_at(base, n);
-    const SingleSource src{sc, r, h, n, nullptr};
+    const DirectSource src{{sc, r, h, n, nullptr}};
     e = cudaMemsetAsync(pb.ctr, 0, kPairCtrWords * sizeof(uint32_t), s);
     if (e == cudaSuccess) {
         if (cfg.mode == kModeAnyHit) {

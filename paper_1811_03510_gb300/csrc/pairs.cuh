@@ -713,7 +713,6 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
     uint32_t pid = 0, start_pid = 0, path = 0, trail = 0;
     RayG<3> pr;
     float tau = 0.0f, c0 = 0.0f, c1 = 0.0f, te = 0.0f;   // intervals are distances from the anchored origin
-    float d[3] = {0.0f, 0.0f, 0.0f};
     int level = 0, rd_target = -1, ctop = 0, cvalid = 0;
     float g[48];
 
@@ -857,8 +856,6 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
                 for (int c = 0; c < 3; ++c) o3[c] = wr.org[c] - pick(c, an.x, an.y, an.z);
                 tau = pair_tau(o3);
             }
-#pragma unroll
-            for (int k = 0; k < 3; ++k) d[k] = 0.0f;
             level = 0;
             rd_target = -1;
             path = trail = 0u;
@@ -941,6 +938,7 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
                         ++level;
                     }
                 } else {
+                    float d[3] = {0.0f, 0.0f, 0.0f};   // displacement of the upper bound (Gregory)
                     if (gpend) {   // Algorithm 2 with the crop of Algorithm 1 for the Gregory node (path, level)
                         float u0, u1, v0, v1;
                         node_domain(path, level, L, u0, u1, v0, v1);
@@ -1155,7 +1153,6 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
                     for (int k = 0; k < 3; ++k) {
                         pr.org[k] = x_pr[k];
                         pr.inv[k] = x_pr[3 + k];
-                        d[k] = 0.0f;
                     }
                     tau = x_tau;
                     te = x_te;

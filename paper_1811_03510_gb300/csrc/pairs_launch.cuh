@@ -55,9 +55,9 @@ cudaError_t launch_pair_passes(const Src &src, const PairBufs &pb, const LaunchC
                   : launch_pair_pass<false, 2, MODE, Src>(src, pb, cfg, n, status, num_sms, s);
 }
 
-cudaError_t pair_passes_single_plain(const SingleSource &src, const PairBufs &pb, const LaunchCfg &cfg, uint32_t n,
+cudaError_t pair_passes_single_plain(const DirectSource &src, const PairBufs &pb, const LaunchCfg &cfg, uint32_t n,
                                      uint32_t *status, int num_sms, cudaStream_t s);
-cudaError_t pair_passes_single_anyhit(const SingleSource &src, const PairBufs &pb, const LaunchCfg &cfg, uint32_t n,
+cudaError_t pair_passes_single_anyhit(const DirectSource &src, const PairBufs &pb, const LaunchCfg &cfg, uint32_t n,
                                       uint32_t *status, int num_sms, cudaStream_t s);
 cudaError_t pair_passes_batch(const BatchSource &src, const PairBufs &pb, const LaunchCfg &cfg, uint32_t n,
                               uint32_t *status, int num_sms, cudaStream_t s);
