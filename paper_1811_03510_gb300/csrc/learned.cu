@@ -318,62 +318,6 @@ __global__ void k_publish_bf16(const float *__restrict__ params, MlpWeights *out
 // Measured on GB300, 450,000 rows: 47 us (161 MB: 3.4 TB/s, half of the measured copy bandwidth), before 97 us (each
 // activation through shared memory, scalar loads and stores).
 // ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16 *p)
-{
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(a));
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
-{
-    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t *>(&v);
-}
-
-// Two row tiles through one layer of 16 KS inputs: acc[m] = bias + A[m] W^T.
-template <int KS>
-__device__ __forceinline__ void infer_layer(const uint32_t (&a)[2][KS][4], const __nv_bfloat16 *W, int stride,
-                                            const float *bias, float (&acc)[2][8][4], int lane)
-{
-    const int t = lane & 3;
-    const __nv_bfloat16 *wl = W + (lane & 7) * stride + 8 * (lane >> 3);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const float bl = bias[8 * j + 2 * t], bh = bias[8 * j + 2 * t + 1];
-#pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            acc[m][j][0] = acc[m][j][2] = bl;
-            acc[m][j][1] = acc[m][j][3] = bh;
-        }
-#pragma unroll
-        for (int ks = 0; ks < KS; ks += 2) {
-            uint32_t b[4];
-            ldmatrix4(b, wl + 8 * j * stride + 16 * ks);
-#pragma unroll
-            for (int m = 0; m < 2; ++m) mma_bf16_16816(acc[m][j], a[m][ks], b[0], b[1]);
-#pragma unroll
-            for (int m = 0; m < 2; ++m) mma_bf16_16816(acc[m][j], a[m][ks + 1], b[2], b[3]);
-        }
-    }
-}
-
-// ReLU and rounding to BF16 of a layer's result, as the A fragments of the next layer.
-__device__ __forceinline__ void relu_fragments(const float (&acc)[2][8][4], uint32_t (&a)[2][4][4])
-{
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int r = 0; r < 2; ++r)
-                    a[m][ks][2 * h + r] =
-                        pack_bf16(fmaxf(acc[m][2 * ks + h][2 * r], 0.0f), fmaxf(acc[m][2 * ks + h][2 * r + 1], 0.0f));
-}
-
 __device__ __forceinline__ float2 load2(const float *p, bool wide)
 {
     return wide ? __ldcs(reinterpret_cast<const float2 *>(p)) : make_float2(__ldcs(p), __ldcs(p + 1));
@@ -417,11 +361,11 @@ __global__ void __launch_bounds__(128, 3) k_mlp_infer(const MlpWeights *__restri
         if (tile + step < tiles) load(tile + step);
         float acc[2][8][4];
         uint32_t a[2][4][4];
-        infer_layer<2>(a1, W.w1, kW1Stride, W.bias, acc, lane);
-        relu_fragments(acc, a);
-        infer_layer<4>(a, W.w2, kW2Stride, W.bias + kHid, acc, lane);
-        relu_fragments(acc, a);
-        infer_layer<4>(a, W.w3, kW2Stride, W.bias + 2 * kHid, acc, lane);
+        mlp_layer<2, 2>(a1, W.w1, kW1Stride, W.bias, acc, lane);
+        relu_fragments<2>(acc, a);
+        mlp_layer<2, 4>(a, W.w2, kW2Stride, W.bias + kHid, acc, lane);
+        relu_fragments<2>(acc, a);
+        mlp_layer<2, 4>(a, W.w3, kW2Stride, W.bias + 2 * kHid, acc, lane);
 #pragma unroll
         for (int m = 0; m < 2; ++m)
 #pragma unroll

@@ -27,11 +27,10 @@ struct MlpWeights {
     float bias[3 * kHid];
 };
 
-// Per-warp tiles for one inference round of 16 rows (32 rows in two rounds).
+// Per-warp tiles of the traversal's inference rounds: the features of 32 lanes (16 rows per round) and the results.
+// The hidden layers stay in registers.
 struct MlpWarpTiles {
     __nv_bfloat16 x[32 * kXStride];
-    __nv_bfloat16 h1[16 * kW2Stride];
-    __nv_bfloat16 h2[16 * kW2Stride];
     uint8_t cell[32];
     float pmax[32];
 };
@@ -60,28 +59,62 @@ __device__ __forceinline__ void load_a(uint32_t (&a)[4], const __nv_bfloat16 *ti
     a[3] = ld_u32(tile + (g + 8) * stride + k0 + 8 + 2 * t);
 }
 
-// One dense layer over 16 rows: out = relu(in . W^T + b) stored as BF16 (STORE) or kept in acc.
-template <int KSTEPS, bool STORE>
-__device__ __forceinline__ void mlp_layer(const __nv_bfloat16 *in, int in_stride, const __nv_bfloat16 *W,
-                                          int w_stride, const float *bias, __nv_bfloat16 *out, float (&acc)[8][4],
-                                          int g, int t)
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16 *p)
 {
-    uint32_t a[KSTEPS][4];
-#pragma unroll
-    for (int ks = 0; ks < KSTEPS; ++ks) load_a(a[ks], in, in_stride, 16 * ks, g, t);
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a));
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
+{
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+
+// M tiles of 16 rows through one layer of 16 KS inputs: acc[m] = bias + A[m] W^T (W in shared memory).
+template <int M, int KS>
+__device__ __forceinline__ void mlp_layer(const uint32_t (&a)[M][KS][4], const __nv_bfloat16 *W, int stride,
+                                          const float *bias, float (&acc)[M][8][4], int lane)
+{
+    const int t = lane & 3;
+    const __nv_bfloat16 *wl = W + (lane & 7) * stride + 8 * (lane >> 3);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const float bl = bias[8 * j + 2 * t], bh = bias[8 * j + 2 * t + 1];
-        acc[j][0] = bl; acc[j][1] = bh; acc[j][2] = bl; acc[j][3] = bh;
-        const __nv_bfloat16 *wrow = W + (8 * j + g) * w_stride;
 #pragma unroll
-        for (int ks = 0; ks < KSTEPS; ++ks)
-            mma_bf16_16816(acc[j], a[ks], ld_u32(wrow + 16 * ks + 2 * t), ld_u32(wrow + 16 * ks + 8 + 2 * t));
-        if (STORE) {
-            st_bf16x2(out + g * kW2Stride + 8 * j + 2 * t, fmaxf(acc[j][0], 0.0f), fmaxf(acc[j][1], 0.0f));
-            st_bf16x2(out + (g + 8) * kW2Stride + 8 * j + 2 * t, fmaxf(acc[j][2], 0.0f), fmaxf(acc[j][3], 0.0f));
+        for (int m = 0; m < M; ++m) {
+            acc[m][j][0] = acc[m][j][2] = bl;
+            acc[m][j][1] = acc[m][j][3] = bh;
+        }
+#pragma unroll
+        for (int ks = 0; ks < KS; ks += 2) {
+            uint32_t b[4];
+            ldmatrix4(b, wl + 8 * j * stride + 16 * ks);
+#pragma unroll
+            for (int m = 0; m < M; ++m) mma_bf16_16816(acc[m][j], a[m][ks], b[0], b[1]);
+#pragma unroll
+            for (int m = 0; m < M; ++m) mma_bf16_16816(acc[m][j], a[m][ks + 1], b[2], b[3]);
         }
     }
+}
+
+// ReLU and rounding to BF16 of a layer's result, as the A fragments of the next layer: the accumulators of two column
+// tiles (m16n8) are the operand of one k-step (m16k16) as they stand.
+template <int M>
+__device__ __forceinline__ void relu_fragments(const float (&acc)[M][8][4], uint32_t (&a)[M][4][4])
+{
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+                    a[m][ks][2 * h + r] =
+                        pack_bf16(fmaxf(acc[m][2 * ks + h][2 * r], 0.0f), fmaxf(acc[m][2 * ks + h][2 * r + 1], 0.0f));
 }
 
 // Argmax (ties: the lowest) and softmax normaliser, sum of exp(v - max), of row h (0 or 1) of a quad's result tile over
@@ -111,23 +144,28 @@ __device__ __forceinline__ void quad_argmax(const float (&acc)[8][4], int h, int
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
 }
 
+// A call, not inlined: in the traversal's loop its fragments would push the ray's state out of registers on every path
+// (1280 x 720 image: 1560 us inlined, 1457 us called).
 // Forward pass of rows [16*r, 16*r+16) of the warp's x tile; writes argmax cell and max softmax
 // probability per row into the tiles (ties: lowest cell).
-__device__ __forceinline__ void mlp_round(const MlpWeights &W, MlpWarpTiles &T, int r, int lane)
+static __device__ __noinline__ void mlp_round(const MlpWeights &W, MlpWarpTiles &T, int r, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
-    float acc[8][4];
-    mlp_layer<2, true>(T.x + 16 * r * kXStride, kXStride, W.w1, kW1Stride, W.bias, T.h1, acc, g, t);
-    __syncwarp();
-    mlp_layer<4, true>(T.h1, kW2Stride, W.w2, kW2Stride, W.bias + kHid, T.h2, acc, g, t);
-    __syncwarp();
-    mlp_layer<4, false>(T.h2, kW2Stride, W.w3, kW2Stride, W.bias + 2 * kHid, nullptr, acc, g, t);
+    float acc[1][8][4];
+    uint32_t a1[1][2][4], a[1][4][4];
+    load_a(a1[0][0], T.x + 16 * r * kXStride, kXStride, 0, g, t);
+    load_a(a1[0][1], T.x + 16 * r * kXStride, kXStride, 16, g, t);
+    mlp_layer<1, 2>(a1, W.w1, kW1Stride, W.bias, acc, lane);
+    relu_fragments<1>(acc, a);
+    mlp_layer<1, 4>(a, W.w2, kW2Stride, W.bias + kHid, acc, lane);
+    relu_fragments<1>(acc, a);
+    mlp_layer<1, 4>(a, W.w3, kW2Stride, W.bias + 2 * kHid, acc, lane);
     // argmax and softmax normaliser of rows g and g + 8 over the quad's 64 columns
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         float best, sum;
         int bidx;
-        quad_argmax(acc, h, t, best, bidx, sum);
+        quad_argmax(acc[0], h, t, best, bidx, sum);
         const int row = 16 * r + g + 8 * h;
         if (t == 0) {
             T.cell[row] = (uint8_t)bidx;

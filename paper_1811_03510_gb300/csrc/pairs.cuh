@@ -924,7 +924,8 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
                     const int last = tab_levels(lsc) - 1;
                     for (;;) {
                         if (STATS) cnt.v[2]++;
-                        so = table_step(nodes + 3 * (size_t)((1u << level) - 1u + path), pr, c0, c1, te, best.t, G, tau);
+                        so = table_step(nodes + 3 * (size_t)((1u << level) - 1u + path), pr, c0, c1, te, best.t, true,
+                                        true, -1, G, tau);
                         if (level == last || iters == 0 || !(so.hitL || so.hitR)) break;
                         --iters;
                         const uint32_t bit = 1u << level;

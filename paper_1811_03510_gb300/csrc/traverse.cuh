@@ -546,7 +546,7 @@ CCS_DEV StepOut split_step(float (&g)[16 * NC], const RayG<NC> &r, const float (
 
 // The same step for a Gregory node whose child boxes are in the scene's table (nd: its 3 float4).
 CCS_DEV StepOut table_step(const float4 *__restrict__ nd, const RayG<3> &r, float c0, float c1, float te, float tb,
-                           const Grp &G, float tau)
+                           bool allowL, bool allowR, int force, const Grp &G, float tau)
 {
     float lmin[3], lmax[3], rmin[3], rmax[3];
 #pragma unroll
@@ -566,11 +566,16 @@ CCS_DEV StepOut table_step(const float4 *__restrict__ nd, const RayG<3> &r, floa
     }
     StepOut o;
     o.dL = o.dR = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        o.dL = __fadd_rn(o.dL, __fsub_rn(lmax[c], lmin[c]));
+        o.dR = __fadd_rn(o.dR, __fsub_rn(rmax[c], rmin[c]));
+    }
     slab<3>(r, lmin, lmax, c0, c1, G, o.l0, o.l1);
     slab<3>(r, rmin, rmax, c0, c1, G, o.r0, o.r1);
-    o.hitL = o.l0 <= o.l1 && __fadd_rn(te, o.l0) <= tb;
-    o.hitR = o.r0 <= o.r1 && __fadd_rn(te, o.r0) <= tb;
-    o.goR = o.hitR && (!o.hitL || o.r0 < o.l0);
+    o.hitL = allowL && o.l0 <= o.l1 && __fadd_rn(te, o.l0) <= tb;
+    o.hitR = allowR && o.r0 <= o.r1 && __fadd_rn(te, o.r0) <= tb;
+    o.goR = force >= 0 ? force == 1 : (o.hitR && (!o.hitL || o.r0 < o.l0));
     return o;
 }
 CCS_DEV const float4 *table_nodes(const DevScene &sc, uint32_t pid)
@@ -977,13 +982,19 @@ CCS_DEV int pair_step(Lane<NC> &s, float (&g)[16 * NC], BvhStack &stk, const Dev
                        const Scratch &scr, Counters &cnt, const ModeCtx &mc, const Grp &G)
 {
     if (MODE == kModeLearned && s.phase == kPhasePropose) return kStepNone;   // waits for the network round
-    if (s.gpend) {   // Algorithm 2 with the crop of Algorithm 1 for the Gregory node (path, level), then
-                     // its split in the same step: a Gregory ray advances one level per warp iteration
+    // A Gregory node whose boxes are in the scene's table.  The learned traversal takes them from there (1280 x 720
+    // image: 1695 -> 1560 us); in the plain one the branch cost scenes with few Gregory patches 2-5% (24,576 patches,
+    // 1283 x 717: 3017 -> 3060 us), though it saved 30% where a quarter are (96 patches: 419 -> 289 us).
+    constexpr bool kTable = MODE == kModeLearned && NC == 3;
+    bool tabled = false;
+    if constexpr (kTable) tabled = s.gpend && s.level < table_levels(sc, L);
+    if (s.gpend && !tabled) {   // Algorithm 2 with the crop of Algorithm 1 for the Gregory node (path, level), then
+                                // its split in the same step: a Gregory ray advances one level per warp iteration
         float u0, u1, v0, v1;
         node_domain(s.path, s.level, L, u0, u1, v0, v1);
         gregory_node<NC>(rec_of(sc, s.pid), u0, u1, v0, v1, s.level, G, g, s.d);
-        s.gpend = false;
     }
+    s.gpend = false;
     const bool redesc = s.rd_target >= 0;
     const bool directed = MODE == kModeLearned && s.phase == kPhaseDirected;
     if (!redesc && (s.level == 2 * L || (MODE == kModeScreen && s.sleaf))) {
@@ -1009,8 +1020,18 @@ CCS_DEV int pair_step(Lane<NC> &s, float (&g)[16 * NC], BvhStack &stk, const Dev
         if ((s.skip_path >> s.level) & 1u) allowR = false; else allowL = false;
     }
     if (STATS && !redesc) cnt.v[s.greg ? 2 : 1]++;
-    const StepOut o = split_step<K, NC>(g, s.pr, s.d, s.c0, s.c1, s.te, s.best.t, redesc || !s.greg, scr, slot,
-                                        allowL, allowR, force, G, s.tau);
+    StepOut o;
+    bool split = true;
+    if constexpr (kTable) {
+        if (tabled) {
+            split = false;
+            o = table_step(table_nodes(sc, s.pid) + 3 * (size_t)((1u << s.level) - 1u + (s.path & ((1u << s.level) - 1u))), s.pr,
+                           s.c0, s.c1, s.te, s.best.t, allowL, allowR, force, G, s.tau);
+        }
+    }
+    if (split)
+        o = split_step<K, NC>(g, s.pr, s.d, s.c0, s.c1, s.te, s.best.t, redesc || !s.greg, scr, slot, allowL, allowR, force,
+                              G, s.tau);
     if (redesc) {
         if (++s.level == s.rd_target) s.rd_target = -1;
         return kStepSplit;

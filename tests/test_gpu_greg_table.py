@@ -86,3 +86,20 @@ def test_table_follows_updates_of_the_points():
     ccs.ccs_batch_destroy(b)
     flat.close()
     sc.close()
+
+
+@pytest.mark.parametrize("depth", [3, 7, 8, 9])
+def test_learned_traversal_with_the_table(depth):
+    """The directed descent and the skipped subtree of the learned order, over table nodes (14 levels) and below."""
+    P, types = gregory_scene(2)
+    r = sg.random_rays(6001, seed=70 + depth, target=1.05)
+    rays = ccs.rays_to_device(r.soa())
+    sc = ccs.Scene(P, types, local=True)
+    ref = trace(sc, rays, r.n, leaf_depth=depth, chunk=32)
+    p = ccs.ccs_proposal_create(seed=6)   # untrained: its cells are arbitrary
+    hits = ccs.alloc_hits(r.n)
+    ccs.ccs_intersect_learned(sc.handle, p, rays, r.n, hits, ccs.make_opts(leaf_depth=depth), 0.0)
+    torch.cuda.synchronize()
+    same(ccs.hits_to_numpy(hits), ref, depth)
+    ccs.ccs_proposal_destroy(p)
+    sc.close()
