@@ -1079,18 +1079,20 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
             }
             waiting = false;
             in_pair = false;
+            if (MODE == kModeAnyHit && best.pid != kMissId) cur = __float_as_uint(rs[13 * stride]);   // answered
             if (hcap[threadIdx.x]) {   // a subtree reached the iteration cap: answered as a capped ray
                 hcap[threadIdx.x] = 0;
                 iters = 0;
                 in_pair = true;
             }
         }
-        // (4) once the queue is empty, idle lanes take a pending subtree of a busy lane of the warp
-        //     (closest-hit mode): the deepest one when its grid is in the busy lane's sibling cache or the
-        //     patch is a Gregory patch (no re-descent), else the shallowest one of at least
-        //     kMinDonateLevels levels (re-descended); the key of a pair's best leaf is the minimum over its
-        //     subtrees
-        if (MODE == kModePlain && exhausted) {
+        // (4) once the queue is empty, idle lanes take a pending subtree of a busy lane of the warp: the
+        //     deepest one when its grid is in the busy lane's sibling cache or the patch is a Gregory patch
+        //     (no re-descent), else the shallowest one of at least kMinDonateLevels levels (re-descended); the
+        //     key of a pair's best leaf is the minimum over its subtrees.  (In the any-hit query too: a ray
+        //     that meets nothing searches as much as a closest-hit ray; 300 k shadow rays on 1,632 patches 350 ->
+        //     266 us.)
+        if (exhausted) {
             const bool idle_l = !has_task && !in_pair;
             const int lmin = trail != 0u ? __ffs(trail) - 1 : 2 * L;
             const int ldeep = trail != 0u ? 31 - __clz(trail) : 2 * L;
