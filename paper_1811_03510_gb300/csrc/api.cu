@@ -43,43 +43,44 @@ static const uint32_t kMaxPatches = 1u << 26;
 
 namespace {
 
-void free_table(GregTabStore &t)
-{
-    cudaFree(t.node);
-    cudaFree(t.rank);
-    cudaFree(t.list);
-    cudaFree(t.depth);
-    t = GregTabStore{};
-}
-
-// Storage of the Gregory box table, within 1/32 of the free device memory; a scene without it (no Gregory patch,
-// no room) has no levels.  The depth word exists in either case.
-cudaError_t alloc_table(ccs_scene *sc)
+// Storage of the Gregory box table, one block: the depth word, the ranks, the list, the nodes.  The nodes take at most
+// 1/32 of the free device memory; a scene without them (no Gregory patch, no room) has no levels, but a depth word.
+cudaError_t alloc_table(ccs_scene *sc, cudaStream_t s)
 {
     GregTabStore &t = sc->tab;
-    cudaError_t e = cudaMalloc(&t.depth, sizeof(uint32_t));
-    if (e != cudaSuccess) return e;
-    if ((e = cudaMemset(t.depth, 0, sizeof(uint32_t))) != cudaSuccess || sc->n_greg == 0) return e;
-    size_t room = 0, total = 0;
-    if ((e = cudaMemGetInfo(&room, &total)) != cudaSuccess) return e;
-    const uint32_t stride = greg_table_levels(sc->n_greg, room / 32);
-    if (stride == 0) return cudaSuccess;
-    std::vector<uint32_t> rank(sc->n), list;
-    list.reserve(sc->n_greg);
-    for (uint32_t p = 0; p < sc->n; ++p) {
-        rank[p] = (uint32_t)list.size();
-        if (sc->htypes[p]) list.push_back(p);
+    uint32_t stride = 0;
+    if (sc->n_greg) {
+        size_t room = 0, total = 0;
+        const cudaError_t e = cudaMemGetInfo(&room, &total);
+        if (e != cudaSuccess) return e;
+        stride = greg_table_levels(sc->n_greg, room / 32);
     }
-    if (cudaMalloc(&t.node, ((size_t)sc->n_greg << stride) * 48) != cudaSuccess ||
-        cudaMalloc(&t.rank, rank.size() * 4) != cudaSuccess || cudaMalloc(&t.list, list.size() * 4) != cudaSuccess) {
+    const size_t n_rank = stride ? sc->n : 0, n_list = stride ? sc->n_greg : 0;
+    const size_t words = (32 + n_rank + n_list + 31) / 32 * 32;   // 128-byte aligned, as the nodes' lines are
+    size_t bytes = words * 4 + (stride ? ((size_t)sc->n_greg << stride) * 64 : 0);
+    cudaError_t e = cudaMalloc(&sc->d_table, bytes);
+    if (e != cudaSuccess && stride) {   // no room after all
         (void)cudaGetLastError();
-        return cudaSuccess;
+        stride = 0;
+        e = cudaMalloc(&sc->d_table, words * 4);
     }
-    if ((e = cudaMemcpy(t.rank, rank.data(), rank.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-    if ((e = cudaMemcpy(t.list, list.data(), list.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
+    uint32_t *w = static_cast<uint32_t *>(sc->d_table);
+    t.depth = w;
+    if (!stride) return cudaMemsetAsync(w, 0, 4, s);
+    std::vector<uint32_t> head(32 + n_rank + n_list, 0u);
+    uint32_t r = 0;
+    for (uint32_t p = 0; p < sc->n; ++p) {
+        head[32 + p] = r;
+        if (sc->htypes[p]) head[32 + n_rank + r++] = p;
+    }
+    if ((e = cudaMemcpyAsync(w, head.data(), head.size() * 4, cudaMemcpyHostToDevice, s)) != cudaSuccess) return e;
+    t.rank = w + 32;
+    t.list = t.rank + n_rank;
+    t.node = reinterpret_cast<float4 *>(w + words);
     t.n = sc->n_greg;
     t.stride = stride;
-    return cudaSuccess;
+    return cudaStreamSynchronize(s);   // (head is read until then)
 }
 
 void free_scene(ccs_scene *s)
@@ -88,7 +89,7 @@ void free_scene(ccs_scene *s)
     cudaFree(s->d_rec);
     cudaFree(s->d_leaf_box);
     cudaFree(s->d_types);
-    free_table(s->tab);
+    cudaFree(s->d_table);
     cudaFree(s->d_nodes);
     cudaFree(s->d_leaf_parent);
     cudaFree(s->d_refit_flags);
@@ -390,7 +391,7 @@ ccs_status ccs_scene_create(ccs_scene **out, const float *x, const float *y, con
             cudaMemcpyAsync(sc->d_types, sc->htypes.data(), n_patches, cudaMemcpyHostToDevice, s);
             e = launch_repack(tmp, tmp + np, tmp + 2 * np, sc->d_types, n_patches, sc->local ? 1 : 0, sc->d_rec,
                               sc->d_leaf_box, s);
-            if (e == cudaSuccess) e = alloc_table(sc);
+            if (e == cudaSuccess) e = alloc_table(sc, s);
             if (e == cudaSuccess) e = launch_greg_table(sc->tab, sc->d_rec, false, s);
             cudaError_t e2 = cudaStreamSynchronize(s);
             cudaFree(tmp);

@@ -67,8 +67,9 @@ struct LaunchCfg {
 
 // Box table of a scene's Gregory patches (table.cu): the child boxes of every node above level `depth` of their
 // subdivision, so that a traversal loads a node's boxes instead of computing Algorithm 2's bound for every ray
-// that visits it.  A node (level l, path p) is 3 float4 at 3 ((rank << stride) + 2^l - 1 + p), axis by axis (lower
-// child lo, hi, upper child lo, hi): the boxes that split_step computes, before the extension of local frames.
+// that visits it.  Node h of a patch (1 the root, 2 h and 2 h + 1 the lower and upper child of h) is 4 float4 at
+// 4 ((rank << stride) + h), axis by axis (lower child lo, hi, upper child lo, hi; the fourth unused): the boxes that
+// split_step computes, before the extension of local frames.  Two siblings share a 128-byte line.
 struct GregTab {
     const float4 *node;
     const uint32_t *rank;    // per patch: its rank among the Gregory patches
@@ -179,7 +180,8 @@ struct ccs_scene {
     float4 *d_leaf_box = nullptr;      // 2 float4 per patch: (lo.xyz, 0), (hi.xyz, 0)
     uint8_t *d_types = nullptr;
     uint32_t n_greg = 0;               // Gregory patches
-    ccs::GregTabStore tab{};           // their box table (no levels when its memory could not be had)
+    void *d_table = nullptr;           // their box table: one block, whose parts tab holds (no levels when the
+    ccs::GregTabStore tab{};           // memory could not be had)
     float4 *d_nodes = nullptr;
     int *d_leaf_parent = nullptr;      // per patch: (node << 1) | slot
     uint32_t *d_refit_flags = nullptr; // per node arrival counters of the refit

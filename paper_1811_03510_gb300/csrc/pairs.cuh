@@ -922,9 +922,17 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
                     // and two slab tests per level, while the others split
                     const float4 *nodes = table_nodes(src.scene(lsc), pid);
                     const int last = tab_levels(lsc) - 1;
+                    uint32_t h = table_index(level, path);
+                    // a step takes less time than a load: each step asks for the lines of the nodes two levels
+                    // down (four nodes, two lines), the first one also for those of one level down
+                    if (level < last) prefetch_l1(nodes + 8 * (size_t)h);
                     for (;;) {
+                        if (level + 1 < last) {
+                            prefetch_l1(nodes + 16 * (size_t)h);
+                            prefetch_l1(nodes + 16 * (size_t)h + 8);
+                        }
                         if (STATS) cnt.v[2]++;
-                        so = table_step(nodes + 3 * (size_t)((1u << level) - 1u + path), pr, c0, c1, te, best.t, true,
+                        so = table_step(nodes + 4 * (size_t)h, pr, c0, c1, te, best.t, true,
                                         true, -1, G, tau);
                         if (level == last || iters == 0 || !(so.hitL || so.hitR)) break;
                         --iters;
@@ -936,6 +944,7 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
                         path = so.goR ? (path | bit) : path;
                         c0 = so.goR ? so.r0 : so.l0;
                         c1 = so.goR ? so.r1 : so.l1;
+                        h = 2 * h + (so.goR ? 1u : 0u);
                         ++level;
                     }
                 } else {

@@ -6,12 +6,13 @@
 //
 // Why: a Gregory step takes a lone warp about 7,000 cycles, a Bezier step 1,600, and a ray that grazes a Gregory patch
 // takes dozens of them one after another, so launches ended on such rays.  A table step (48 bytes, two slab tests)
-// is bound by the latency of its load.  Measured, before and after (us per pair-engine call): 64 x 64 rays on 96
-// patches 165 -> 129, 330 k diffuse rays on 1,632 patches 250 -> 220, 300 k any-hit shadow rays there 536 -> 410, 1.2 M
-// mirror rays on 98,400 patches 665 -> 565; 1080p primary rays, which rarely meet one, unchanged.
-// Levels: meshes have few irregular faces, so their tables may be deep; 14 levels (786 KB) per patch while they fit in
-// 128 MB.  (16, all of leaf depth 8: 120 us instead of 129 on the 96 patches, but scene creation took 0.3 ms
-// longer, 14%.)  After an update of the points 10 levels, built beside the batch's refit: no time of its own.
+// is bound by the latency of its load, so two siblings share a line and each step asks for the lines of the nodes two
+// levels down.  Measured, before and after (us per pair-engine call): 64 x 64 rays on 96 patches 165 -> 115, 330 k
+// diffuse rays on 1,632 patches 250 -> 191, 1.2 M mirror rays on 98,400 patches 665 -> 525; 1080p primary rays, which
+// rarely meet one, unchanged.  (The prefetches and the siblings' shared lines: 214 -> 202 us on the diffuse rays.)
+// Levels: meshes have few irregular faces, so their tables may be deep; 16 levels, all of leaf depth 8 (4.2 MB), per
+// patch while they fit in 256 MB (14 levels: 149 us instead of 132 on 96 patches of another seed).  After an update of
+// the points 10 levels, built beside the batch's refit: no time of its own.
 #include <algorithm>
 
 #include "table_dev.cuh"
@@ -35,7 +36,7 @@ uint32_t greg_table_levels(uint32_t n, size_t bytes)
 {
     const uint64_t most = std::min<uint64_t>(bytes, kGregBytes);
     uint32_t D = n ? kGregLevels : 0;
-    while (D > 0 && ((uint64_t)n << D) * 48 > most) --D;
+    while (D > 0 && ((uint64_t)n << D) * 64 > most) --D;
     return D;
 }
 

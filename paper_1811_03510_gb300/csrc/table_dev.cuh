@@ -6,8 +6,8 @@
 namespace ccs {
 
 // levels stored; levels built after an update of the points (an animated scene pays for the build every frame)
-constexpr uint32_t kGregLevels = 14, kGregUpdateLevels = 10;
-constexpr uint64_t kGregBytes = (uint64_t)128 << 20;
+constexpr uint32_t kGregLevels = 16, kGregUpdateLevels = 10;
+constexpr uint64_t kGregBytes = (uint64_t)256 << 20;
 
 __host__ __device__ inline uint32_t greg_update_levels(uint32_t stored) { return stored < kGregUpdateLevels ? stored : kGregUpdateLevels; }
 
@@ -24,7 +24,7 @@ CCS_DEV void greg_table_node(const GregTabStore &t, const float4 *__restrict__ r
     SplitPts<3> S;
     float lmin[3], lmax[3], rmin[3], rmax[3];
     split_boxes<3>(g, d, S, lmin, lmax, rmin, rmax);
-    float4 *nd = t.node + 3 * (((size_t)rank << t.stride) + m);
+    float4 *nd = t.node + 4 * (((size_t)rank << t.stride) + table_index(level, path));
 #pragma unroll
     for (int k = 0; k < 3; ++k) nd[k] = make_float4(lmin[k], lmax[k], rmin[k], rmax[k]);
 }

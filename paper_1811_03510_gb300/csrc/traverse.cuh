@@ -544,7 +544,7 @@ CCS_DEV StepOut split_step(float (&g)[16 * NC], const RayG<NC> &r, const float (
     return o;
 }
 
-// The same step for a Gregory node whose child boxes are in the scene's table (nd: its 3 float4).
+// The same step for a Gregory node whose child boxes are in the scene's table (at nd).
 CCS_DEV StepOut table_step(const float4 *__restrict__ nd, const RayG<3> &r, float c0, float c1, float te, float tb,
                            bool allowL, bool allowR, int force, const Grp &G, float tau)
 {
@@ -578,10 +578,12 @@ CCS_DEV StepOut table_step(const float4 *__restrict__ nd, const RayG<3> &r, floa
     o.goR = force >= 0 ? force == 1 : (o.hitR && (!o.hitL || o.r0 < o.l0));
     return o;
 }
-CCS_DEV const float4 *table_nodes(const DevScene &sc, uint32_t pid)
+CCS_DEV const float4 *table_nodes(const DevScene &sc, uint32_t pid)   // node h at 4 h
 {
-    return sc.tab.node + 3 * ((size_t)__ldg(sc.tab.rank + pid) << sc.tab.stride);
+    return sc.tab.node + 4 * ((size_t)__ldg(sc.tab.rank + pid) << sc.tab.stride);
 }
+CCS_DEV uint32_t table_index(int level, uint32_t path) { return level ? (1u << level) | (__brev(path) >> (32 - level)) : 1u; }
+CCS_DEV void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 // The levels of Gregory pairs whose boxes are in the scene's table.
 CCS_DEV int table_levels(const DevScene &sc, int L) { return min((int)__ldg(sc.tab.depth), 2 * L); }
 
@@ -1025,8 +1027,7 @@ CCS_DEV int pair_step(Lane<NC> &s, float (&g)[16 * NC], BvhStack &stk, const Dev
     if constexpr (kTable) {
         if (tabled) {
             split = false;
-            o = table_step(table_nodes(sc, s.pid) + 3 * (size_t)((1u << s.level) - 1u + (s.path & ((1u << s.level) - 1u))), s.pr,
-                           s.c0, s.c1, s.te, s.best.t, allowL, allowR, force, G, s.tau);
+            o = table_step(table_nodes(sc, s.pid) + 4 * (size_t)table_index(s.level, s.path & ((1u << s.level) - 1u)), s.pr, s.c0, s.c1, s.te, s.best.t, allowL, allowR, force, G, s.tau);
         }
     }
     if (split)

@@ -40,7 +40,7 @@ def gregory_scene(n):
     return P.astype(np.float32), types
 
 
-# 96 patches hold 14 levels, 1536 patches 10 (128 MiB): leaf depths 1..9 lie above, at and below them
+# 96 patches hold 15 levels, 1536 patches 11 (256 MiB): leaf depths 1..9 lie above, at and below them
 @pytest.mark.parametrize("local", [False, True])
 @pytest.mark.parametrize("n,depth", [(2, 1), (2, 3), (2, 7), (2, 8), (2, 9), (8, 4), (8, 5), (8, 6)])
 def test_table_hits_equal_the_ray_kernel(n, depth, local):
@@ -90,7 +90,7 @@ def test_table_follows_updates_of_the_points():
 
 @pytest.mark.parametrize("depth", [3, 7, 8, 9])
 def test_learned_traversal_with_the_table(depth):
-    """The directed descent and the skipped subtree of the learned order, over table nodes (14 levels) and below."""
+    """The directed descent and the skipped subtree of the learned order, over table nodes (15 levels) and below."""
     P, types = gregory_scene(2)
     r = sg.random_rays(6001, seed=70 + depth, target=1.05)
     rays = ccs.rays_to_device(r.soa())
