@@ -138,10 +138,11 @@ typedef struct {
                                        pair engine. */
 #define CCS_TRACE_PAIRS 8u          /* pair engine, for the plain closest hit and the any-hit query with one
                                        lane per ray (other modes ignore it): (1) one thread per ray walks
-                                       the BVH and keeps the ray's 8 nearest candidate patches (by entry
-                                       distance of the patch box); with local frames a Bezier patch whose
-                                       root box in its own frame the ray does not come near is no
-                                       candidate; (2) the rays with candidates are ordered by a cost
+                                       the BVH (warps with coherent rays walk it once for all of them) and
+                                       keeps the ray's 8 nearest candidate patches (by entry distance of
+                                       the patch box); a Bezier patch whose root box in its own frame,
+                                       without local frames padded by the size of a leaf box, the ray does
+                                       not come near is no candidate; (2) the rays with candidates are ordered by a cost
                                        class (a Gregory candidate first, then more candidates first);
                                        (3) persistent warps run Algorithm 3 on one (ray, patch) pair per
                                        lane, taking each ray's candidates in entry order until one enters
@@ -157,7 +158,8 @@ typedef struct {
                                        listed, rays that dropped some, walks for dropped candidates,
                                        subtrees handed over, warp iterations of the subdivision pass and,
                                        per iteration, lanes splitting, helping, waiting and idle, then
-                                       candidates culled by their root box. */
+                                       candidates culled by their root box with local frames; slot 18 those
+                                       culled without. */
 #define CCS_NUM_COUNTERS 23         /* work per ray, summed (0..7): bvh nodes, bezier splits, gregory
                                        splits, leaves, backtracks, re-descent levels, pruned siblings, pairs;
                                        schedule of the warps, summed over warp iterations (8..19): warp

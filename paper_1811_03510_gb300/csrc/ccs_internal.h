@@ -17,7 +17,8 @@ namespace ccs {
 //   [0..3] x of the 16 grid slots (slot 4*j + i), [4..7] y, [8..11] z,
 //   [12] x of p^v (inner slots (1,1),(2,1),(1,2),(2,2)), [13] y, [14] z,
 //   [15] anchor xyz (world box centre), w = 1 for Gregory, 0 for Bezier,
-//   [16..18] rows of the frame (identity without local frames), [19] unused.
+//   [16..18] rows of the patch's frame, w: low corner of a Bezier patch's root box in it, [19] its high corner, w: with
+//   local frames 1 + the L1 diagonal of that box, without them the size bound of a leaf box at leaf depth 0.
 constexpr int kRecF4 = 20;
 
 // BVH node = 4 float4 = 64 bytes (both children's boxes stored in the parent), one float4 per axis so

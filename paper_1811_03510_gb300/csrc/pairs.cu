@@ -78,7 +78,7 @@ cudaError_t launch_cand(const Src &src, const PairBufs &pb, const LaunchCfg &cfg
     const uint32_t img_w = (cfg.image_width & 7u) == 0u ? cfg.image_width : 0u;
     const uint32_t t = cand_threads(n, img_w);
     k_cand<STATS, MODE, Src, BW><<<(t + kCandBlock - 1) / kCandBlock, kCandBlock, 0, s>>>(
-        src, pb, img_w, cfg.iter_cap, status, cfg.counters, cfg.mc.occluded);
+        src, pb, img_w, (int)cfg.leaf_depth, cfg.iter_cap, status, cfg.counters, cfg.mc.occluded);
     return cudaGetLastError();
 }
 

@@ -3,9 +3,8 @@
 //  1. k_cand: one thread per ray walks the BVH (Sec. 4) and keeps the ray's kPairCands nearest candidate
 //     patches, ordered by (entry distance of the patch box, patch id).  Before the list is full nothing
 //     is pruned but [tmin, tmax]; once it is full, subtrees that enter beyond its last entry are skipped
-//     and the smallest entry distance dropped that way is kept (t_evict).  With local frames a Bezier patch
-//     whose root box in its own frame the ray does not come near is no candidate (root_box_near: its pair
-//     would end at the first split).  A ray with candidates becomes a task with a cost class (the highest when a candidate is a Gregory patch, else its number of
+//     and the smallest entry distance dropped that way is kept (t_evict).  A Bezier patch whose root box in its
+//     own frame the ray does not come near is no candidate (root_box_near: its pair would record no leaf).  A ray with candidates becomes a task with a cost class (the highest when a candidate is a Gregory patch, else its number of
 //     candidates); rays with no candidate are written as misses here.
 //  2. Each task's index goes to the list of its cost class (the candidate pass counts the classes' places),
 //     and the subdivision pass's queue takes the classes costliest first, so that the long rays start
@@ -140,23 +139,30 @@ CCS_DEV void write_miss(const Src &src, uint32_t scene, uint32_t j, uint8_t *occ
     }
 }
 
-// Cull test of a candidate with local frames (Sec. 3.4): does the ray pass near the patch's root box in
-// the patch frame?  Every box of a Bezier pair's subdivision lies in that box (de Casteljau midpoints stay
-// between their operands), widened by the box extension by at most tau / 2; a pair's FP32 slab tests
-// report a hit only within about 1e-6 (|o - anchor| + box diagonal) of a box.  The test pads the box by
-// 2^-16 (1 + |o - anchor|_1 + |hi - lo|_1), far more than both and far less than a patch, so a culled
-// pair holds no leaf that its subdivision would record.  Gregory patches are kept (their boxes come from
-// the bounds of Algorithm 2, not from the control points).
+// Cull test of a candidate: does the ray pass near the patch's root box in the patch's own frame (Sec. 3.4)?  With
+// local frames every box of a Bezier pair's subdivision lies in that box (de Casteljau midpoints stay between their
+// operands), widened by the box extension by at most tau / 2.  Without them the boxes are world boxes, but what a pair
+// records are leaves, and a leaf's box reaches at most its own size beyond the points inside the root box
+// (leaf = 2^-L: at most leaf times the bound in slot 19).  A pair's FP32 slab tests report a hit only within about
+// 1e-6 (|o - anchor| + box diagonal) of a box; the test pads the box by 2^-16 (1 + |o - anchor|_1 + |hi - lo|_1),
+// far more than that and far less than a patch, and by the leaf's size, so a culled pair holds no leaf that its
+// subdivision would record.  Gregory patches are kept (their boxes come from the bounds of Algorithm 2, not from the
+// control points).
+// Without local frames this measured (1283 x 717 images, binary BVH): candidates 699 k -> 385 k and rays with more than
+// the list holds 15,090 -> 2 on 1,536 patches, so that no lane ends the launch walking the BVH again; call 813 -> 628 us,
+// on 24,576 patches 1714 -> 1131 us, 153 k bounce rays there 746 -> 310 us.
 CCS_DEV bool root_box_near(const float4 *__restrict__ rec, const float (&o)[3], const float (&d)[3], float tmin,
-                           const Grp &G)
+                           bool local, float leaf, const Grp &G)
 {
     const float4 an = __ldg(rec + 15);
     if (an.w != 0.0f) return true;
     const float4 R[3] = {__ldg(rec + 16), __ldg(rec + 17), __ldg(rec + 18)};
     const float4 hb = __ldg(rec + 19);
     const float o3[3] = {__fsub_rn(o[0], an.x), __fsub_rn(o[1], an.y), __fsub_rn(o[2], an.z)};
-    const float pad = __fmul_rn(__int_as_float((127 - 16) << 23),
-                                __fadd_rn(hb.w, __fadd_rn(__fadd_rn(fabsf(o3[0]), fabsf(o3[1])), fabsf(o3[2]))));
+    const float diag1 = local ? hb.w : 1.0f + ((hb.x - R[0].w) + (hb.y - R[1].w) + (hb.z - R[2].w));
+    float pad = __fmul_rn(__int_as_float((127 - 16) << 23),
+                          __fadd_rn(diag1, __fadd_rn(__fadd_rn(fabsf(o3[0]), fabsf(o3[1])), fabsf(o3[2]))));
+    if (!local) pad = fmaf(leaf, hb.w, pad);
     RayG<3> r;
     float lo[3], hi[3];
 #pragma unroll
@@ -174,15 +180,14 @@ CCS_DEV bool root_box_near(const float4 *__restrict__ rec, const float (&o)[3], 
 // ------------------------------------------------------------------------------------------------
 // Pass 1: BVH walk with the sorted candidate list.
 // ------------------------------------------------------------------------------------------------
-// A patch whose box the ray enters at n0: into the sorted list, unless (local frames, Bezier) the ray does not come
-// near its root box; the last entry of a full list, or the patch itself, is dropped.
+// A patch whose box the ray enters at n0: into the sorted list, unless the ray does not come near its root box; the last entry of a full list, or the patch itself, is dropped.
 template <bool STATS>
 CCS_DEV void list_patch(const DevScene &sc, uint32_t p, float n0, const float (&ro)[3], const float (&rd)[3], float tmin,
-                        float (&kt)[kPairCands], uint32_t (&kp)[kPairCands], int &cnt, float &t_evict, bool &evicted,
+                        float leaf, float (&kt)[kPairCands], uint32_t (&kp)[kPairCands], int &cnt, float &t_evict, bool &evicted,
                         unsigned long long &culled, const Grp &G)
 {
     constexpr int C = kPairCands;
-    if (sc.local && !root_box_near(rec_of(sc, p), ro, rd, tmin, G)) {
+    if (!root_box_near(rec_of(sc, p), ro, rd, tmin, sc.local != 0, leaf, G)) {
         if (STATS) ++culled;
         return;
     }
@@ -212,12 +217,12 @@ CCS_DEV void list_patch(const DevScene &sc, uint32_t p, float n0, const float (&
 // distance of the patch box, patch id), sorted in kt / kp, counting only keys above (lb_t, lb_p) when has_lb
 // (the candidates an earlier walk did not list: all its dropped keys are above its last listed one).  Before
 // the list is full nothing is pruned but [tmin, tmax]; once it is full, subtrees entered beyond its last
-// entry are skipped and the smallest entry distance dropped that way is kept (t_evict).  With local frames,
-// Bezier patches whose root box the ray does not come near are no candidates (root_box_near).  Returns false
-// when the iteration budget it ran out.
+// entry are skipped and the smallest entry distance dropped that way is kept (t_evict).  Bezier patches
+// whose root box the ray does not come near are no candidates (root_box_near).  Returns false when the iteration budget
+// it ran out.
 template <bool STATS, int BW>
 CCS_DEV bool walk_candidates(const DevScene &sc, const RayG<3> &r, const float (&ro)[3], const float (&rd)[3],
-                             float tmin, float tmax, bool has_lb, float lb_t, uint32_t lb_p, uint32_t &it,
+                             float tmin, float tmax, float leaf, bool has_lb, float lb_t, uint32_t lb_p, uint32_t &it,
                              float (&kt)[kPairCands], uint32_t (&kp)[kPairCands], int &cnt, float &t_evict,
                              bool &evicted, unsigned long long &nodes, unsigned long long &culled, const Grp &G)
 {
@@ -234,7 +239,7 @@ CCS_DEV bool walk_candidates(const DevScene &sc, const RayG<3> &r, const float (
             const uint32_t p = (uint32_t)(~node);
             // (not one that an earlier walk listed)
             if (!has_lb || cand_less(lb_t, lb_p, n0, p))
-                list_patch<STATS>(sc, p, n0, ro, rd, tmin, kt, kp, cnt, t_evict, evicted, culled, G);
+                list_patch<STATS>(sc, p, n0, ro, rd, tmin, leaf, kt, kp, cnt, t_evict, evicted, culled, G);
         } else {
             ++nodes;
             // once the list is full, a subtree entered beyond its last entry only holds dropped patches
@@ -469,7 +474,7 @@ inline uint32_t cand_threads(uint32_t n, uint32_t img_w)
 }
 
 template <bool STATS, int MODE, class Src, int BW>
-__global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint32_t img_w, uint32_t iter_cap,
+__global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint32_t img_w, int L, uint32_t iter_cap,
                                               uint32_t *status, unsigned long long *counters, uint8_t *occluded)
 {
     const unsigned FULL = 0xffffffffu;
@@ -477,7 +482,7 @@ __global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint3
     const uint32_t n = src.total();
     const uint32_t i = cand_ray(blockIdx.x * blockDim.x + threadIdx.x, img_w);
     constexpr int C = kPairCands;
-    const float kInf = __int_as_float(0x7f800000);
+    const float kInf = __int_as_float(0x7f800000), leaf = __int_as_float((127 - L) << 23);
     float kt[C];
     uint32_t kp[C];
 #pragma unroll
@@ -530,11 +535,11 @@ __global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint3
                 const float lo[3] = {blo.x, blo.y, blo.z}, hi[3] = {bhi.x, bhi.y, bhi.z};
                 float t0, t1;
                 slab<3>(r, lo, hi, tmin, tmax, G, t0, t1);
-                if (t0 <= t1) list_patch<STATS>(sc, p, t0, ro, rd, tmin, kt, kp, cnt, t_evict, evicted, culled, G);
+                if (t0 <= t1) list_patch<STATS>(sc, p, t0, ro, rd, tmin, leaf, kt, kp, cnt, t_evict, evicted, culled, G);
             }
         } else if (ok) {
             uint32_t it = iter_cap;
-            capped = !walk_candidates<STATS, BW>(sc, r, ro, rd, tmin, tmax, false, 0.0f, 0u, it, kt, kp, cnt, t_evict,
+            capped = !walk_candidates<STATS, BW>(sc, r, ro, rd, tmin, tmax, leaf, false, 0.0f, 0u, it, kt, kp, cnt, t_evict,
                                                  evicted, nodes, culled, G);
         }
     }
@@ -580,15 +585,19 @@ __global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint3
     }
     if (STATS) {   // BVH nodes; diagnostics in the schedule slots: candidates listed, rays that dropped some,
                    // candidates culled by their root box
-        unsigned long long v[4] = {nodes, want, (unsigned long long)(has && evicted), culled};
+        // (those culled where the boxes are world boxes in a slot of their own)
+        const bool world = live && src.scene(lsc).local == 0;
+        unsigned long long v[5] = {nodes, want, (unsigned long long)(has && evicted), world ? 0ull : culled,
+                                   world ? culled : 0ull};
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < 5; ++k)
             for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(FULL, v[k], o);
         if (lane == 0) {
             if (v[0]) atomicAdd(counters + 0, v[0]);
             if (v[1]) atomicAdd(counters + 8, v[1]);
             if (v[2]) atomicAdd(counters + 9, v[2]);
             if (v[3]) atomicAdd(counters + 17, v[3]);
+            if (v[4]) atomicAdd(counters + 18, v[4]);
         }
     }
 }
@@ -603,7 +612,7 @@ struct MoreCands {
     bool evicted, capped;
 };
 template <int BW>
-__device__ __forceinline__ MoreCands collect_more(const DevScene sc, const float *rs, int stride, float lb_t,
+__device__ __forceinline__ MoreCands collect_more(const DevScene sc, const float *rs, int stride, float leaf, float lb_t,
                                                uint32_t lb_p, uint32_t iter_cap, uint2 *dst)
 {
     constexpr int C = kPairCands;
@@ -632,7 +641,7 @@ __device__ __forceinline__ MoreCands collect_more(const DevScene sc, const float
     G.mask = 0xffffffffu;
     G.l0 = G.l1 = G.l2 = threadIdx.x & 31;
     uint32_t it = iter_cap;
-    out.capped = !walk_candidates<false, BW>(sc, r, ro, rd, rs[6 * stride], rs[7 * stride], true, lb_t, lb_p, it, kt, kp,
+    out.capped = !walk_candidates<false, BW>(sc, r, ro, rd, rs[6 * stride], rs[7 * stride], leaf, true, lb_t, lb_p, it, kt, kp,
                                              out.cnt, out.t_evict, out.evicted, nodes, culled, G);
     if (!out.capped)
         for (int j = 0; j < out.cnt; ++j) dst[j] = make_uint2(kp[j], __float_as_uint(kt[j]));
@@ -737,8 +746,8 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
                         const DevScene &sc = src.scene(lsc);
                         const MoreCands mc =
                             sc.width == 4
-                                ? collect_more<4>(sc, rs, stride, __uint_as_float(last.y), last.x, iter_cap, pb.cand + cbase)
-                                : collect_more<2>(sc, rs, stride, __uint_as_float(last.y), last.x, iter_cap, pb.cand + cbase);
+                                ? collect_more<4>(sc, rs, stride, cellw, __uint_as_float(last.y), last.x, iter_cap, pb.cand + cbase)
+                                : collect_more<2>(sc, rs, stride, cellw, __uint_as_float(last.y), last.x, iter_cap, pb.cand + cbase);
                         if (STATS) cnt.v[10]++;
                         evicted = mc.evicted;
                         if (mc.capped) {   // iteration cap of the walk: a miss, status latched

@@ -72,15 +72,39 @@ __device__ __forceinline__ void repack_one(const float *__restrict__ x, const fl
             r[12 + c] = make_float4(comp(c, 16), comp(c, 17), comp(c, 18), comp(c, 19));
         else
             r[12 + c] = make_float4(comp(c, 5), comp(c, 6), comp(c, 9), comp(c, 10));
-        r[16 + c] = local ? make_float4(R[c][0], R[c][1], R[c][2], 0.0f)
-                          : make_float4(c == 0 ? 1.0f : 0.0f, c == 1 ? 1.0f : 0.0f, c == 2 ? 1.0f : 0.0f, 0.0f);
+        r[16 + c] = make_float4(R[c][0], R[c][1], R[c][2], 0.0f);
     }
     r[15] = make_float4(an[0], an[1], an[2], greg ? 1.0f : 0.0f);
     // the root box of a Bezier patch in its own frame: the AABB of the 16 stored grid components, which
     // holds every box of its subdivision (de Casteljau midpoints stay between their operands); lo in
     // the w of the frame rows, hi and 1 + |hi - lo|_1 in slot 19 (Gregory patches: unused, zero)
-    float blo[3] = {0.0f, 0.0f, 0.0f}, bhi[3] = {0.0f, 0.0f, 0.0f};
-    if (!greg) {
+    // (without local frames the boxes of the subdivision are world boxes and the frame serves the cull alone: the root
+    // box of the points in it, and in slot 19 the bound of a leaf's size, three times the L1 norms of the largest
+    // control-point differences along u and along v: the box of a leaf of 2^-L x 2^-L spans at most 2^-L of it)
+    float blo[3] = {0.0f, 0.0f, 0.0f}, bhi[3] = {0.0f, 0.0f, 0.0f}, leaf_size = 0.0f;
+    if (!greg && !local) {
+        for (int k = 0; k < 16; ++k) {
+            const float dx = pl[0][k] - an[0], dy = pl[1][k] - an[1], dz = pl[2][k] - an[2];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float q = fmaf(R[c][0], dx, fmaf(R[c][1], dy, R[c][2] * dz));
+                blo[c] = k ? fminf(blo[c], q) : q;
+                bhi[c] = k ? fmaxf(bhi[c], q) : q;
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            float du = 0.0f, dv = 0.0f;
+            for (int j = 0; j < 4; ++j)
+                for (int k = 0; k < 3; ++k) {
+                    du = fmaxf(du, fabsf(pl[c][4 * j + k + 1] - pl[c][4 * j + k]));
+                    dv = fmaxf(dv, fabsf(pl[c][4 * k + 4 + j] - pl[c][4 * k + j]));
+                }
+            leaf_size += 3.0f * (du + dv);
+            r[16 + c].w = blo[c];
+        }
+    }
+    if (!greg && local) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             float a = r[c * 4].x, b = a;
@@ -95,7 +119,9 @@ __device__ __forceinline__ void repack_one(const float *__restrict__ x, const fl
         }
     }
     r[19] = make_float4(bhi[0], bhi[1], bhi[2],
-                        greg ? 0.0f : 1.0f + ((bhi[0] - blo[0]) + (bhi[1] - blo[1])) + (bhi[2] - blo[2]));
+                        greg     ? 0.0f
+                        : !local ? leaf_size
+                                 : 1.0f + ((bhi[0] - blo[0]) + (bhi[1] - blo[1])) + (bhi[2] - blo[2]));
     leaf_box[2 * (size_t)p] = make_float4(lo[0], lo[1], lo[2], 0.0f);
     leaf_box[2 * (size_t)p + 1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
 }
