@@ -213,16 +213,15 @@ CCS_DEV void list_patch(const DevScene &sc, uint32_t p, float n0, const float (&
     kp[0] = m == 0 ? p : kp[0];
 }
 
-// The BVH walk of the candidate pass (Sec. 4): the C candidates of the ray with the smallest keys (entry
-// distance of the patch box, patch id), sorted in kt / kp, counting only keys above (lb_t, lb_p) when has_lb
-// (the candidates an earlier walk did not list: all its dropped keys are above its last listed one).  Before
-// the list is full nothing is pruned but [tmin, tmax]; once it is full, subtrees entered beyond its last
-// entry are skipped and the smallest entry distance dropped that way is kept (t_evict).  Bezier patches
-// whose root box the ray does not come near are no candidates (root_box_near).  Returns false when the iteration budget
-// it ran out.
+// A BVH walk of one ray (Sec. 4): the C candidates of the ray with the smallest keys (entry distance of the patch box,
+// patch id) above (lb_t, lb_p), sorted in kt / kp: those that an earlier walk did not list (all its dropped keys are
+// above its last listed one).  Before the list is full nothing is pruned but [tmin, tmax]; once it is full, subtrees
+// entered beyond its last entry are skipped and the smallest entry distance dropped that way is kept (t_evict).  Bezier
+// patches whose root box the ray does not come near are no candidates (root_box_near).  Returns false when the
+// iteration budget it ran out.
 template <bool STATS, int BW>
 CCS_DEV bool walk_candidates(const DevScene &sc, const RayG<3> &r, const float (&ro)[3], const float (&rd)[3],
-                             float tmin, float tmax, float leaf, bool has_lb, float lb_t, uint32_t lb_p, uint32_t &it,
+                             float tmin, float tmax, float leaf, float lb_t, uint32_t lb_p, uint32_t &it,
                              float (&kt)[kPairCands], uint32_t (&kp)[kPairCands], int &cnt, float &t_evict,
                              bool &evicted, unsigned long long &nodes, unsigned long long &culled, const Grp &G)
 {
@@ -238,7 +237,7 @@ CCS_DEV bool walk_candidates(const DevScene &sc, const RayG<3> &r, const float (
         if (node < 0) {   // a patch: into the list (the leaf's box is the patch box)
             const uint32_t p = (uint32_t)(~node);
             // (not one that an earlier walk listed)
-            if (!has_lb || cand_less(lb_t, lb_p, n0, p))
+            if (cand_less(lb_t, lb_p, n0, p))
                 list_patch<STATS>(sc, p, n0, ro, rd, tmin, leaf, kt, kp, cnt, t_evict, evicted, culled, G);
         } else {
             ++nodes;
@@ -344,6 +343,99 @@ CCS_DEV bool walk_candidates(const DevScene &sc, const RayG<3> &r, const float (
         }
     }
     return true;
+}
+
+// The walk of one ray in the candidate pass: the kPairCands nearest of all its candidates.  Patches go to a buffer of the
+// lane in shared memory (buf, strided), and are looked at together once a lane's buffer is full or its walk done: the
+// lanes of a warp, out of step in the tree, then share the expensive part (the cull, 5 loads, and the insertion), and the
+// node loop holds nothing else.  The children are not sorted, but the nearest is entered first: the order only decides
+// what a full list drops.
+// Measured (us per call, walking node by node and patch by patch before): 1.2 M mirror rays on 98,400 patches 527 -> 492,
+// 330 k diffuse rays on 1,632 patches 190 -> 177, 4K image of 98,304 patches (warps without a beam) 1761 -> 1753; with a
+// buffer of 4 patches 569 / 185 / 1866, of 8 506 / 179 / 1775, of 16 490 / 176 / 1750 but 1410 instead of 1376 us for an
+// animated batch (shared memory).
+constexpr int kLeafBuf = 12;
+template <bool STATS, int BW>
+CCS_DEV bool walk_buffered(const DevScene &sc, const RayG<3> &r, const float (&ro)[3], const float (&rd)[3], float tmin,
+                           float tmax, float leaf, uint32_t &it, float (&kt)[kPairCands], uint32_t (&kp)[kPairCands],
+                           int &cnt, float &t_evict, bool &evicted, unsigned long long &nodes, unsigned long long &culled,
+                           uint2 *buf, int stride, const Grp &G)
+{
+    constexpr int C = kPairCands;
+    int stk[kBvhStack];
+    int sp = 0, node = 0, nb = 0;
+    for (;;) {
+        while (node != kDone && nb <= kLeafBuf - BW) {
+            if (it == 0) return false;
+            --it;
+            ++nodes;
+            // once the list is full, a subtree entered beyond its last entry only holds dropped patches
+            const float bound = cnt == C ? kt[C - 1] : __int_as_float(0x7f800000);
+            int next = kDone;
+            float next_t = 0.0f;
+            auto child = [&](int c, float t0, float t1) {
+                if (!(t0 <= t1) || c == kEmptyChild) return;
+                if (t0 > bound) {
+                    evicted = true;
+                    t_evict = fminf(t_evict, t0);
+                } else if (c < 0) {
+                    buf[nb * stride] = make_uint2((uint32_t)(~c), __float_as_uint(t0));
+                    ++nb;
+                } else {
+                    int far = c;
+                    if (next == kDone || t0 < next_t) {
+                        far = next;
+                        next = c;
+                        next_t = t0;
+                    }
+                    if (far != kDone && sp < kBvhStack) stk[sp++] = far;
+                }
+            };
+            if constexpr (BW == 4) {
+                const float4 *nd = sc.nodes + (size_t)node * kNode4F4;
+                float4 lo4[3], hi4[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    lo4[k] = __ldg(nd + 2 * k);
+                    hi4[k] = __ldg(nd + 2 * k + 1);
+                }
+                const int4 ch = __ldg(reinterpret_cast<const int4 *>(nd + 6));
+                const int c[4] = {ch.x, ch.y, ch.z, ch.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    float lo[3], hi[3];
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        lo[k] = j == 0 ? lo4[k].x : j == 1 ? lo4[k].y : j == 2 ? lo4[k].z : lo4[k].w;
+                        hi[k] = j == 0 ? hi4[k].x : j == 1 ? hi4[k].y : j == 2 ? hi4[k].z : hi4[k].w;
+                    }
+                    float t0, t1;
+                    slab<3>(r, lo, hi, tmin, tmax, G, t0, t1);
+                    child(c[j], t0, t1);
+                }
+            } else {
+                const float4 *nd = sc.nodes + (size_t)node * kNodeF4;
+                float4 q[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) q[k] = __ldg(nd + k);
+                const int2 ch = __ldg(reinterpret_cast<const int2 *>(nd + 3));
+                float a0, a1, b0, b1;
+                node_child_boxes<3>(q, r, tmin, tmax, G, a0, a1, b0, b1);
+                child(ch.x, a0, a1);
+                child(ch.y, b0, b1);
+            }
+            node = next != kDone ? next : sp > 0 ? stk[--sp] : kDone;
+        }
+#pragma unroll 1
+        for (int q = 0; q < nb; ++q) {
+            if (it == 0) return false;
+            --it;
+            const uint2 e = buf[q * stride];
+            list_patch<STATS>(sc, e.x, __uint_as_float(e.y), ro, rd, tmin, leaf, kt, kp, cnt, t_evict, evicted, culled, G);
+        }
+        nb = 0;
+        if (node == kDone) return true;
+    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -502,6 +594,7 @@ __global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint3
     G.l0 = G.l1 = G.l2 = lane;
     float ro[3] = {0.0f, 0.0f, 0.0f}, rd[3] = {0.0f, 0.0f, 0.0f}, tmin = 0.0f, tmax = 0.0f;
     __shared__ int beam[kCandBlock / 32 * kBeamWords];
+    __shared__ uint2 leaf_buf[kLeafBuf * kCandBlock];
     RayG<3> r;
     bool ok = false;
 #pragma unroll
@@ -539,8 +632,8 @@ __global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint3
             }
         } else if (ok) {
             uint32_t it = iter_cap;
-            capped = !walk_candidates<STATS, BW>(sc, r, ro, rd, tmin, tmax, leaf, false, 0.0f, 0u, it, kt, kp, cnt, t_evict,
-                                                 evicted, nodes, culled, G);
+            capped = !walk_buffered<STATS, BW>(sc, r, ro, rd, tmin, tmax, leaf, it, kt, kp, cnt, t_evict, evicted, nodes,
+                                               culled, leaf_buf + threadIdx.x, kCandBlock, G);
         }
     }
     // the task: the candidates in list order in one run of the buffer; its cost class
@@ -641,7 +734,7 @@ __device__ __forceinline__ MoreCands collect_more(const DevScene sc, const float
     G.mask = 0xffffffffu;
     G.l0 = G.l1 = G.l2 = threadIdx.x & 31;
     uint32_t it = iter_cap;
-    out.capped = !walk_candidates<false, BW>(sc, r, ro, rd, rs[6 * stride], rs[7 * stride], leaf, true, lb_t, lb_p, it, kt, kp,
+    out.capped = !walk_candidates<false, BW>(sc, r, ro, rd, rs[6 * stride], rs[7 * stride], leaf, lb_t, lb_p, it, kt, kp,
                                              out.cnt, out.t_evict, out.evicted, nodes, culled, G);
     if (!out.capped)
         for (int j = 0; j < out.cnt; ++j) dst[j] = make_uint2(kp[j], __float_as_uint(kt[j]));
