@@ -36,6 +36,7 @@ struct SingleSource {
         scene = 0;
         local = perm ? __ldg(perm + i) : i;
     }
+    CCS_DEV bool world_boxes() const { return sc.local == 0; }
     CCS_DEV const DevRays &rays_of(uint32_t) const { return rays; }
     CCS_DEV const DevHits &hits_of(uint32_t) const { return hits; }
 };
@@ -71,6 +72,7 @@ struct BatchSource {
         local = i - __ldg(ray_prefix + lo);
         lsc.s = lo;
     }
+    CCS_DEV bool world_boxes() const { return entries[0].sc.local == 0; }   // (scenes of a batch are mostly alike)
     CCS_DEV const DevRays &rays_of(uint32_t s) const { return entries[s].rays; }
     CCS_DEV const DevHits &hits_of(uint32_t s) const { return entries[s].hits; }
 };

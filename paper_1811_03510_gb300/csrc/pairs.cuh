@@ -768,12 +768,23 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
     hcount[threadIdx.x] = 0;
     hcap[threadIdx.x] = 0;
     // the queue hands out the tasks class by class, costliest first: cstart[c] = first place of class c
-    __shared__ uint32_t cstart[kCostClasses + 1];
+    __shared__ uint32_t cstart[kCostClasses + 1], share[2];
     if (threadIdx.x < kCostClasses) {
         uint32_t a = 0;
         for (int c = kCostClasses - 1; c > (int)threadIdx.x; --c) a += pb.ctr[kCtrHist + c];
         cstart[threadIdx.x] = a;
-        if (threadIdx.x == 0) cstart[kCostClasses] = a + pb.ctr[kCtrHist];   // all tasks
+        if (threadIdx.x == 0) {
+            const uint32_t all = a + pb.ctr[kCtrHist], warps = gridDim.x * (blockDim.x >> 5);
+            cstart[kCostClasses] = all;
+            // A refill takes at most share[0] tasks, so that a short queue is spread over all warps, whose other lanes
+            // help (64 x 64 image: 128 -> 90 us).  Without local frames the first shares of all warps, the costliest
+            // tasks, are dealt out like cards, every share[1]-th task to one warp: neighbours in the list are
+            // neighbours on the surface, grazing rays among them many times longer than the others, and one warp would
+            // hold 32 of them (1283 x 717 image of 1,536 patches 625 -> 477 us).  With local frames no ray is that long,
+            // and what counts is that the rays of a warp share patches (1080p image 422 us, dealt out 443).
+            share[0] = min(32u, max(1u, (all + warps - 1u) / warps));
+            share[1] = src.world_boxes() ? min(warps, all / share[0]) : 0u;
+        }
     }
     __syncthreads();
     Counters cnt;
@@ -788,7 +799,6 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
     G.l0 = G.l1 = G.l2 = lane;
     const float kInf = __int_as_float(0x7f800000);
     const float cellw = __int_as_float((127 - L) << 23);
-    const uint32_t n_tasks = cstart[kCostClasses];
     uint32_t *queue = pb.ctr + kCtrQueue;
     if (STATS && lane == 0) atomicMax(counters + 20, ~global_ns());   // first warp start
 
@@ -883,14 +893,17 @@ __global__ void __launch_bounds__(128, 3) k_pairs(Src src, PairBufs pb, int L, u
             const unsigned idle = __ballot_sync(FULL, !has_task);
             if (idle == 0u || ((uint32_t)__popc(idle) < refill && idle != FULL)) break;
             uint32_t qb = 0;
-            if (lane == 0) qb = atomicAdd(queue, (uint32_t)__popc(idle));
+            const uint32_t take = min(share[0], (uint32_t)__popc(idle));
+            if (lane == 0) qb = atomicAdd(queue, take);
             qb = __shfl_sync(FULL, qb, 0);
-            if (qb + (uint32_t)__popc(idle) >= n_tasks) {
+            if (qb + take >= cstart[kCostClasses]) {
                 exhausted = true;
                 if (STATS && lane == 0) atomicMax(counters + 21, ~global_ns());   // queue found empty
             }
-            const uint32_t k = qb + (uint32_t)__popc(idle & lt);
-            if (!has_task && k < n_tasks) {
+            const uint32_t rank = (uint32_t)__popc(idle & lt);
+            uint32_t k = qb + rank;
+            if (!has_task && rank < take && k < cstart[kCostClasses]) {
+                if (k < share[0] * share[1]) k = k % share[0] * share[1] + k / share[0];
                 int c = kCostClasses - 1;
                 while (c > 0 && k >= cstart[c - 1]) --c;
                 const uint4 *tp = pb.task + 4 * (size_t)__ldg(pb.cls + (size_t)c * pb.n + (k - cstart[c]));

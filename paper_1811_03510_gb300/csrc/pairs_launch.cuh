@@ -32,7 +32,7 @@ cudaError_t launch_pair_pass(const Src &src, const PairBufs &pb, const LaunchCfg
     }
     if (occ_active < 1) return cudaErrorInvalidConfiguration;
     uint32_t blocks = (uint32_t)num_sms * (uint32_t)occ_active;
-    const uint32_t needed = (n + threads - 1) / threads;   // tasks of one kind are at most one per ray
+    const uint32_t needed = (n + 31) / 32;   // a task per warp at least, if every eighth ray has one
     if (blocks > needed) blocks = needed;
     if (blocks == 0) blocks = 1;
     kern<<<blocks, threads, smem, s>>>(src, pb, (int)cfg.leaf_depth, cfg.refill, cfg.iter_cap, status, cfg.counters,
