@@ -14,19 +14,18 @@ bool use_pairs(const LaunchCfg &cfg)
            cfg.lanes_per_ray == 1;
 }
 
-// The engine of a launch that leaves it open, by both engines' times over images and their bounce rays (96 to 98,304
-// patches, 16 x 16 to 1283 x 717 pixels; ray-persistent / pair engine).  World-axis boxes: the pair engine at every
-// size (1283 x 717 image 1484 / 676 us on 1,536 patches, 16 x 16 225 / 170; bounce rays 1.1 to 3.3 times faster, but
-// 0.93 times for 153,000 rays on 24,576 patches or more).  Local frames: from 2^14 rays on (1283 x 717 image 553 / 242
-// us, 256 x 144 1.04 to 1.55 times faster); below, its three launches and its tail cost what it saves (64 x 64 0.87 to
-// 1.11 times, 6,144 bounce rays 0.75 to 1.28).  With the 1-slot sibling cache, its fastest on images.
+// The engine of a launch that leaves it open: the pair engine, by both engines' times over images and their bounce rays
+// (96 to 98,304 patches, 16 x 16 to 1283 x 717 pixels; ray-persistent / pair engine).  World-axis boxes: 1.34 to 5.8 times
+// faster (1283 x 717 image of 1,536 patches 1474 / 450 us, 16 x 16 226 / 118).  Local frames: 1.05 to 3.1 times faster on
+// images (1283 x 717 551 / 243 us, 16 x 16 91 / 71), 0.99 to 2.4 on bounce rays but for 6,144 of them on 98,304 patches
+// (119 / 148 us).  With the 1-slot sibling cache, its fastest on images.
 // Not above 2^23 rays (an 8.3 M pixel image fits), whose scratch of 1.6 GB the library's pool would keep, and not while
 // the stream is captured, where the ray-persistent kernel needs no allocation; that kernel also takes the launch when
 // the scratch cannot be had (launch_intersect).
-void choose_engine(LaunchCfg &cfg, bool local, uint32_t n, cudaStream_t s)
+void choose_engine(LaunchCfg &cfg, uint32_t n, cudaStream_t s)
 {
-    constexpr uint32_t kLeastLocal = 1u << 14, kMostRays = 1u << 23;
-    if (!cfg.auto_engine || n > kMostRays || (local && n < kLeastLocal)) return;
+    constexpr uint32_t kMostRays = 1u << 23;
+    if (!cfg.auto_engine || n > kMostRays) return;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
         (void)cudaGetLastError();
