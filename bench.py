@@ -150,7 +150,10 @@ def whole_job_rate(rays_per_step: int, steps: int, t_slowest: float, world: int)
 def engine_of(o) -> str:
     from paper_1811_03510_gb300 import ccs
     d = ccs.opts_dict(o)
-    return "pairs" if d["pairs"] and d["lanes_per_ray"] != 3 else ("ray+order" if d["order"] else "ray")
+    # options that leave the engine open get the pair engine (include/ccs.h, ccs_trace_opts.flags)
+    open_ = not o.flags and not any(d[k] for k in ("block_threads", "blocks_per_sm", "chunk", "bvh_burst", "min_blocks",
+                                                   "vote")) and not o.iter_cap and not o.pixel_spread
+    return "pairs" if (d["pairs"] or open_) and d["lanes_per_ray"] != 3 else ("ray+order" if d["order"] else "ray")
 
 
 def kernels_per_launch(o) -> int:
