@@ -9,9 +9,26 @@
 #pragma once
 #include <type_traits>
 
+#include "launch_cache.h"
 #include "traverse.cuh"
 
 namespace ccs {
+
+// Resident blocks per SM of a kernel on the current device, its shared memory limit raised to smem before.
+template <class Kernel>
+cudaError_t resident_blocks(LaunchCache &cache, Kernel kern, uint32_t threads, size_t smem, int *active)
+{
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return cache.blocks_per_sm<cudaError_t>(
+        dev, threads, smem,
+        [&](size_t bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); },
+        [&](uint32_t t, size_t bytes, int *a) {
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(a, kern, (int)t, bytes);
+        },
+        active);
+}
 
 // Device clock in nanoseconds (the timeline counters of a counting launch).
 CCS_DEV unsigned long long global_ns()
@@ -300,25 +317,10 @@ static cudaError_t launch_one(const Src &src, const LaunchCfg &cfg, uint32_t *qu
     const uint32_t threads = cfg.block_threads;
     size_t smem = smem_bytes<BW>(threads, cfg.leaf_depth, K, NC);
     if (MODE == kModeLearned) smem += sizeof(MlpWeights) + (threads / 32) * sizeof(MlpWarpTiles);
-    static size_t configured = 0;   // largest dynamic shared memory size set on this instantiation
-    if (smem > configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = smem;
-    }
-    // resident blocks per SM for this instantiation, block size and shared memory (queried once per shape)
-    static uint32_t occ_threads = 0;
-    static size_t occ_smem = 0;
-    static int occ_active = 0;
-    if (occ_threads != threads || occ_smem != smem) {
-        int max_active = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&max_active, kern, (int)threads, smem);
-        if (e != cudaSuccess) return e;
-        occ_threads = threads;
-        occ_smem = smem;
-        occ_active = max_active;
-    }
-    const int max_active = occ_active;
+    static LaunchCache cache;
+    int max_active = 0;
+    const cudaError_t e = resident_blocks(cache, kern, threads, smem, &max_active);
+    if (e != cudaSuccess) return e;
     if (max_active < 1) return cudaErrorInvalidConfiguration;
     uint32_t per_sm = cfg.blocks_per_sm < (uint32_t)max_active ? cfg.blocks_per_sm : (uint32_t)max_active;
     uint32_t blocks = (uint32_t)num_sms * per_sm;

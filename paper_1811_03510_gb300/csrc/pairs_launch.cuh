@@ -15,21 +15,10 @@ cudaError_t launch_pair_pass(const Src &src, const PairBufs &pb, const LaunchCfg
     constexpr uint32_t threads = 128;
     const size_t smem =
         (size_t)threads * (scratch_floats((int)cfg.leaf_depth, K, 3) + kRaySlotFloats + kHelpFloats) * sizeof(float);
-    static size_t configured = 0;   // largest dynamic shared memory size set on this instantiation
-    static size_t occ_smem = 0;
-    static int occ_active = 0;
-    if (smem > configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = smem;
-    }
-    if (occ_smem != smem) {
-        int a = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, kern, (int)threads, smem);
-        if (e != cudaSuccess) return e;
-        occ_smem = smem;
-        occ_active = a;
-    }
+    static LaunchCache cache;
+    int occ_active = 0;
+    const cudaError_t e = resident_blocks(cache, kern, threads, smem, &occ_active);
+    if (e != cudaSuccess) return e;
     if (occ_active < 1) return cudaErrorInvalidConfiguration;
     uint32_t blocks = (uint32_t)num_sms * (uint32_t)occ_active;
     const uint32_t needed = (n + 31) / 32;   // a task per warp at least, if every eighth ray has one
