@@ -107,9 +107,10 @@ typedef struct {
     uint32_t image_width;     /* the rays are an image of this width, ray y * width + x (the last row may
                                  be partial).  CCS_TRACE_ORDER: ordered in tiles of 8 x 8 pixels with
                                  every 4th pixel in x and y sampled; 0: tiles of 32 consecutive rays,
-                                 every 4th ray sampled.  CCS_TRACE_PAIRS, a multiple of 8: each warp of
-                                 the candidate pass takes a tile of 8 x 4 pixels (a host chunk is tiled
-                                 from its own first ray); else 32 consecutive rays.  Never changes the
+                                 every 4th ray sampled.  Pair engine, a multiple of 8 and at most the
+                                 number of rays: each warp of the candidate pass takes a tile of 8 x 4
+                                 pixels (a host chunk is tiled from its own first ray); else 32
+                                 consecutive rays.  Never changes the
                                  answer [0] */
     uint32_t bvh_width;       /* the scene's BVH to traverse: 0 its default, 2 or 4 (INVALID_ARG when the
                                  scene was not built with that width) [0] */
