@@ -181,7 +181,18 @@ CCS_DEV bool root_box_near(const float4 *__restrict__ rec, const float (&o)[3], 
 // ------------------------------------------------------------------------------------------------
 // Pass 1: BVH walk with the sorted candidate list.
 // ------------------------------------------------------------------------------------------------
-// A patch whose box the ray enters at n0: into the sorted list, unless the ray does not come near its root box; the last entry of a full list, or the patch itself, is dropped.
+// Whether root_box_near can tell for a ray with direction d.  safe_inv moves components below 1e-20 to that size, along the
+// world axes for the BVH's boxes and along the frame's axes here, so the two rays agree only where that is nothing: with a
+// largest component of 2^-40 or more it is less than the rounding of the rotated direction.  Up to 2^100 the rotated
+// components and their inverses are finite and normal.
+CCS_DEV bool cullable(const float (&d)[3])
+{
+    const float m = max3f(fabsf(d[0]), fabsf(d[1]), fabsf(d[2]));
+    return m >= __int_as_float((127 - 40) << 23) && m <= __int_as_float((127 + 100) << 23);
+}
+
+// A patch whose box the ray enters at n0: into the sorted list, unless the ray does not come near its root box; the last
+// entry of a full list, or the patch itself, is dropped.
 template <bool STATS>
 CCS_DEV void list_patch(const DevScene &sc, uint32_t p, float n0, const float (&ro)[3], const float (&rd)[3], float tmin,
                         float leaf, float (&kt)[kPairCands], uint32_t (&kp)[kPairCands], int &cnt, float &t_evict, bool &evicted,
@@ -591,6 +602,8 @@ __global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint3
         ro[1] = r.org[1];
         ro[2] = r.org[2];
     }
+    // (a register less than a flag: with a NaN component root_box_near keeps every patch)
+    if (!cullable(rd)) rd[0] = __int_as_float(0x7fffffff);
     const unsigned rays = __ballot_sync(FULL, ok);
     if (rays != 0u) {
         // one walk for the warp, when its rays make a beam (of one scene)
@@ -641,6 +654,7 @@ __global__ void __launch_bounds__(kCandBlock) k_cand(Src src, PairBufs pb, uint3
         for (int j = 0; j < C; ++j)
             if (j < cnt) dst[j] = make_uint2(kp[j], __float_as_uint(kt[j]));
         uint4 *tk = pb.task + 4 * (size_t)i;
+        if (isnan(rd[0])) rd[0] = __ldg(src.rays_of(ray_scene).dx + ray_local);
         tk[0] = make_uint4(i, (uint32_t)off, (uint32_t)cnt | ((uint32_t)key << 8) | (evicted ? kTaskEvicted : 0u),
                            __float_as_uint(t_evict));
         tk[1] = make_uint4(kp[0], __float_as_uint(kt[0]), __float_as_uint(tmin), __float_as_uint(tmax));
@@ -700,6 +714,7 @@ __device__ __forceinline__ MoreCands collect_more(const DevScene sc, const float
         r.inv[k] = rs[(3 + k) * stride];
         rd[k] = rs[(9 + k) * stride];
     }
+    if (!cullable(rd)) rd[0] = __int_as_float(0x7fffffff);
     float kt[C];
     uint32_t kp[C];
 #pragma unroll
