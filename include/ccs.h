@@ -101,8 +101,11 @@ typedef struct {
                                  lanes_per_ray 0 or 1, the library picks the engine: ccs_intersect,
                                  ccs_intersect_host, ccs_intersect_host_batches and ccs_occluded then run
                                  the pair engine (CCS_TRACE_PAIRS, with the 1-slot cache for
-                                 CCS_CACHE_DEFAULT) for up to 2^23 rays outside stream capture while its
-                                 scratch can be had, and the ray-persistent kernel otherwise */
+                                 CCS_CACHE_DEFAULT and refill at most 24) for 32 to 2^23 rays outside
+                                 stream capture while its scratch can be had, but not at leaf depths to 3
+                                 in world axes with up to 16 rays per patch; and the ray-persistent
+                                 kernel, which allocates nothing, otherwise.  An option of that kernel
+                                 written out (chunk = 32, say) asks for it */
     uint64_t *counters;       /* optional device array of CCS_NUM_COUNTERS uint64 (CCS_TRACE_COUNT) */
     uint32_t image_width;     /* the rays are an image of this width, ray y * width + x (the last row may
                                  be partial).  CCS_TRACE_ORDER: ordered in tiles of 8 x 8 pixels with

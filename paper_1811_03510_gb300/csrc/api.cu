@@ -539,7 +539,7 @@ ccs_status ccs_intersect(const ccs_scene *sc, const ccs_rays *rays, uint32_t n, 
     if ((st = fill_launch_cfg(opts, cfg)) != CCS_OK) return st;
     CCS_ARG(has_width(sc, cfg.bvh_width), "the scene has no BVH of the width opts->bvh_width asks for");
     if (cfg.pixel_spread > 0.0f) cfg.mode = 4;   // screen-space termination (one lane per ray)
-    choose_engine(cfg, n, (cudaStream_t)stream);
+    choose_engine(cfg, sc, n, (cudaStream_t)stream);
     DevScene ds = dev_scene(sc, cfg.bvh_width);
     DevRays dr{rays->ox, rays->oy, rays->oz, rays->dx, rays->dy, rays->dz, rays->tmin, rays->tmax};
     DevHits dh{hits->t, hits->u, hits->v, hits->patch_id};
@@ -663,7 +663,7 @@ ccs_status ccs_intersect_host(ccs_scene *sc, const ccs_rays *hr, uint32_t n, ccs
             return CCS_OK;
         }
     }
-    choose_engine(cfg, n, s);
+    choose_engine(cfg, sc, n, s);
     const HostBatch one{hr, n, hh, cfg};
     return host_pipeline(sc, &one, 1, s);
 }
@@ -686,7 +686,7 @@ ccs_status ccs_intersect_host_batches(ccs_scene *sc, uint32_t n_batches, const c
         if ((st = fill_launch_cfg(opts ? opts[j] : nullptr, cfg)) != CCS_OK) return st;
         CCS_ARG(has_width(sc, cfg.bvh_width), "the scene has no BVH of the width opts->bvh_width asks for");
         if (cfg.pixel_spread > 0.0f) cfg.mode = 4;
-        choose_engine(cfg, n[j], (cudaStream_t)stream);
+        choose_engine(cfg, sc, n[j], (cudaStream_t)stream);
         bt[j] = HostBatch{&hr[j], n[j], &hh[j], cfg};
     }
     return host_pipeline(sc, bt.data(), n_batches, (cudaStream_t)stream);
@@ -751,7 +751,7 @@ ccs_status ccs_occluded(const ccs_scene *sc, const ccs_rays *rays, uint32_t n, u
     CCS_ARG(has_width(sc, cfg.bvh_width), "the scene has no BVH of the width opts->bvh_width asks for");
     cfg.mode = 3;
     cfg.mc.occluded = occluded;
-    choose_engine(cfg, n, (cudaStream_t)stream);
+    choose_engine(cfg, sc, n, (cudaStream_t)stream);
     DevScene ds = dev_scene(sc, cfg.bvh_width);
     DevRays dr{rays->ox, rays->oy, rays->oz, rays->dx, rays->dy, rays->dz, rays->tmin, rays->tmax};
     DevHits dh{nullptr, nullptr, nullptr, nullptr};

@@ -145,7 +145,7 @@ cudaError_t launch_intersect_batch(const BatchEntry *entries, const uint32_t *ra
 // launches (single scene: scratch from the library's stream-ordered pool; batch: the caller's scratch)
 bool use_pairs(const LaunchCfg &cfg);
 // the engine of a launch of n rays on stream s whose options leave it open
-void choose_engine(LaunchCfg &cfg, uint32_t n, cudaStream_t s);
+void choose_engine(LaunchCfg &cfg, const ccs_scene *sc, uint32_t n, cudaStream_t s);
 size_t pairs_scratch_bytes(uint32_t n);
 // scratch of one launch from the library's stream-ordered memory pool of the current device (pairs.cu):
 // allocated and freed in the order of `s`; freed memory stays in the pool for reuse

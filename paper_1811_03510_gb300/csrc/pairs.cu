@@ -4,6 +4,7 @@
 // batch, so that its run stays capturable in a CUDA graph.
 #include <mutex>
 
+#include "engine_plan.h"
 #include "pairs_launch.cuh"
 
 namespace ccs {
@@ -14,18 +15,12 @@ bool use_pairs(const LaunchCfg &cfg)
            cfg.lanes_per_ray == 1;
 }
 
-// The engine of a launch that leaves it open: the pair engine, by both engines' times over images and their bounce rays
-// (96 to 98,304 patches, 16 x 16 to 1283 x 717 pixels; ray-persistent / pair engine).  World-axis boxes: 1.34 to 5.8 times
-// faster (1283 x 717 image of 1,536 patches 1474 / 450 us, 16 x 16 226 / 118).  Local frames: 1.05 to 3.1 times faster on
-// images (1283 x 717 551 / 243 us, 16 x 16 91 / 71), 0.99 to 2.4 on bounce rays but for 6,144 of them on 98,304 patches
-// (119 / 148 us).  With the 1-slot sibling cache, its fastest on images.
-// Not above 2^23 rays (an 8.3 M pixel image fits), whose scratch of 1.6 GB the library's pool would keep, and not while
-// the stream is captured, where the ray-persistent kernel needs no allocation; that kernel also takes the launch when
-// the scratch cannot be had (launch_intersect).
-void choose_engine(LaunchCfg &cfg, uint32_t n, cudaStream_t s)
+// The engine of a launch that leaves it open: by its size (engine_plan.h), with the 1-slot sibling cache, the pair engine's
+// fastest on images.  Not while the stream is captured, where the ray-persistent kernel needs no allocation; that kernel
+// also takes the launch when the scratch cannot be had (launch_intersect).
+void choose_engine(LaunchCfg &cfg, const ccs_scene *sc, uint32_t n, cudaStream_t s)
 {
-    constexpr uint32_t kMostRays = 1u << 23;
-    if (!cfg.auto_engine || n > kMostRays) return;
+    if (!cfg.auto_engine || !pairs_by_default(n, sc->n, sc->local, cfg.leaf_depth)) return;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -33,6 +28,7 @@ void choose_engine(LaunchCfg &cfg, uint32_t n, cudaStream_t s)
     }
     if (cap != cudaStreamCaptureStatusNone) return;
     cfg.flags |= CCS_TRACE_PAIRS;
+    cfg.refill = default_pairs_refill(cfg.refill);
     if (cfg.auto_cache) cfg.cache_slots = 1;
 }
 
