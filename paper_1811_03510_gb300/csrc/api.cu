@@ -11,6 +11,7 @@
 #include "bvh_build.h"
 #include "ccs_internal.h"
 #include "host_plan.h"
+#include "table_plan.h"
 
 namespace ccs {
 

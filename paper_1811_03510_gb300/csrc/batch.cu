@@ -4,6 +4,7 @@
 // and no synchronisation, so it can be captured into a CUDA graph (ccs_batch_capture).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <new>
 #include <string>
@@ -90,15 +91,15 @@ static cudaError_t launch_batch_table_refit(const BatchEntry *entries, const uin
                                             uint32_t n_greg, uint32_t levels, uint32_t *flags, uint32_t n_flag_words,
                                             cudaStream_t s)
 {
-    if (n_greg == 0 || levels == 0)
+    if (n_greg == 0)
         return flags ? launch_batch_refit(entries, patch_prefix, n_scenes, n_patches, flags, n_flag_words, s) : cudaSuccess;
     if (flags) {
         cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(uint32_t) * n_flag_words, s);
         if (e != cudaSuccess) return e;
     }
-    const uint32_t D = greg_update_levels(levels), refit_blocks = flags ? (n_patches + 127) / 128 : 0;
-    const size_t blocks = refit_blocks + (((size_t)n_greg << D) + 127) / 128;
-    k_batch_table_refit<<<(unsigned)blocks, 128, 0, s>>>(entries, patch_prefix, greg_prefix, n_scenes, n_patches, n_greg, D,
+    const uint32_t refit_blocks = flags ? (n_patches + 127) / 128 : 0;
+    const size_t blocks = refit_blocks + (((size_t)n_greg << levels) + 127) / 128;
+    k_batch_table_refit<<<(unsigned)blocks, 128, 0, s>>>(entries, patch_prefix, greg_prefix, n_scenes, n_patches, n_greg, levels,
                                                          refit_blocks);
     return cudaGetLastError();
 }
@@ -116,7 +117,7 @@ struct ccs_batch {
     BatchEntry *d_table = nullptr;
     uint32_t *d_ray_prefix = nullptr, *d_patch_prefix = nullptr;
     uint32_t *d_greg_prefix = nullptr;    // Gregory patches of the scenes that have a box table for them
-    uint32_t n_greg = 0, greg_levels = 0; // their number; the levels of the deepest table
+    uint32_t n_greg = 0, greg_levels = 0; // their number; the most levels that an update builds
     uint32_t *d_flags = nullptr;          // refit arrival counters of every scene's nodes
     uint32_t *d_work = nullptr;           // [0] queue head, [1] status word
     void *d_pairs = nullptr;              // the pair engine's scratch (CCS_TRACE_PAIRS), made on first use
@@ -228,7 +229,7 @@ ccs_status ccs_batch_create(ccs_batch **out, ccs_scene *const *scenes, uint32_t 
             pp[s] = p;
             gp[s] = b->n_greg;
             b->n_greg += sc->tab.n;
-            if (sc->tab.stride > b->greg_levels) b->greg_levels = sc->tab.stride;
+            b->greg_levels = std::max(b->greg_levels, greg_update_levels(sc->tab.n, sc->tab.stride));
             r += n_rays[s];
             p += sc->n;
             nn += sc->n_nodes;

@@ -124,9 +124,8 @@ struct BatchEntry {
 // kernels (intersect.cu, scene.cu)
 cudaError_t launch_repack(const float *x, const float *y, const float *z, const uint8_t *types, uint32_t n, int local,
                           float4 *rec, float4 *leaf_box, cudaStream_t s);
-// Gregory box tables (table.cu): the levels that `bytes` hold for n patches; the build after a repack (every
-// level, or after an update of the points fewer; a batch builds them beside its refit)
-uint32_t greg_table_levels(uint32_t n, size_t bytes);
+// Gregory box tables (table.cu): the build after a repack (every level, or after an update of the points fewer; a batch
+// builds them beside its refit)
 cudaError_t launch_greg_table(const GregTabStore &t, const float4 *rec, bool update, cudaStream_t s);
 cudaError_t launch_refit(float4 *nodes, const int *leaf_parent, const float4 *leaf_box, uint32_t *flags,
                          uint32_t n_patches, uint32_t n_nodes, uint32_t width, cudaStream_t s);

@@ -12,9 +12,7 @@
 // rarely meet one, unchanged.  (The prefetches and the siblings' shared lines: 214 -> 202 us on the diffuse rays.)
 // Levels: meshes have few irregular faces, so their tables may be deep; 16 levels, all of leaf depth 8 (4.2 MB), per
 // patch while they fit in 256 MB (14 levels: 149 us instead of 132 on 96 patches of another seed).  After an update of
-// the points 10 levels, built beside the batch's refit: no time of its own.
-#include <algorithm>
-
+// the points at most 10 levels and 2^16 nodes (table_plan.h), built beside a batch's refit.
 #include "table_dev.cuh"
 
 namespace ccs {
@@ -32,19 +30,11 @@ __global__ void __launch_bounds__(128) k_greg_table(GregTabStore t, const float4
 
 }  // namespace
 
-uint32_t greg_table_levels(uint32_t n, size_t bytes)
-{
-    const uint64_t most = std::min<uint64_t>(bytes, kGregBytes);
-    uint32_t D = n ? kGregLevels : 0;
-    while (D > 0 && ((uint64_t)n << D) * 64 > most) --D;
-    return D;
-}
-
 cudaError_t launch_greg_table(const GregTabStore &t, const float4 *rec, bool update, cudaStream_t s)
 {
     if (!t.stride) return cudaSuccess;
-    const uint32_t D = update ? greg_update_levels(t.stride) : t.stride;
-    const size_t n = (size_t)t.n << D;
+    const uint32_t D = update ? greg_update_levels(t.n, t.stride) : t.stride;
+    const size_t n = D ? (size_t)t.n << D : 1;   // (no level: the depth word alone)
     k_greg_table<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(t, rec, D);
     return cudaGetLastError();
 }

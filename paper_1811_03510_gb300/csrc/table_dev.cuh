@@ -1,15 +1,10 @@
 // Device routines of the Gregory box tables (described in table.cu), shared by its kernels and the batch's refit.
 #pragma once
 
+#include "table_plan.h"
 #include "traverse.cuh"
 
 namespace ccs {
-
-// levels stored; levels built after an update of the points (an animated scene pays for the build every frame)
-constexpr uint32_t kGregLevels = 16, kGregUpdateLevels = 10;
-constexpr uint64_t kGregBytes = (uint64_t)256 << 20;
-
-__host__ __device__ inline uint32_t greg_update_levels(uint32_t stored) { return stored < kGregUpdateLevels ? stored : kGregUpdateLevels; }
 
 // Node m of 2^D - 1 (level by level) of the Gregory patch of the given rank.
 CCS_DEV void greg_table_node(const GregTabStore &t, const float4 *__restrict__ rec, uint32_t rank, uint32_t m)
@@ -42,9 +37,10 @@ CCS_DEV void batch_greg_node(const BatchEntry *__restrict__ entries, const uint3
         if (__ldg(prefix + h) <= p) lo = h; else hi = h;
     }
     const BatchEntry &e = entries[lo];
-    const uint32_t rank = p - prefix[lo], D = greg_update_levels(e.tab.stride);
-    if (!e.px || m + 1u >= (1u << D)) return;
+    const uint32_t rank = p - prefix[lo], D = greg_update_levels(e.tab.n, e.tab.stride);
+    if (!e.px) return;
     if (rank == 0 && m == 0) *e.tab.depth = D;
+    if (m + 1u >= (1u << D)) return;
     greg_table_node(e.tab, e.rec, rank, m);
 }
 
