@@ -4,7 +4,6 @@
 // and no synchronisation, so it can be captured into a CUDA graph (ccs_batch_capture).
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <cstring>
 #include <new>
 #include <string>
@@ -36,35 +35,50 @@ __global__ void k_batch_repack(const BatchEntry *__restrict__ entries, const uin
     repack_one(e.px, e.py, e.pz, e.types, gp - patch_prefix[s], e.rec, e.leaf_box, (int)e.sc.local);
 }
 
-__global__ void k_batch_refit(const BatchEntry *__restrict__ entries, const uint32_t *__restrict__ patch_prefix,
-                              uint32_t n_scenes, uint32_t n_patches)
+__device__ __forceinline__ void batch_refit_patch(const BatchEntry *__restrict__ entries,
+                                                  const uint32_t *__restrict__ patch_prefix, uint32_t n_scenes,
+                                                  uint32_t n_patches, uint32_t gp)
 {
-    const uint32_t gp = blockIdx.x * blockDim.x + threadIdx.x;
     if (gp >= n_patches) return;
     const uint32_t s = find_scene(patch_prefix, n_scenes, gp);
     const BatchEntry &e = entries[s];
     refit_one(e.nodes, e.leaf_parent, e.leaf_box, e.refit_flags, gp - patch_prefix[s], e.sc.width);
 }
 
-// Gregory box tables of the scenes with new points, and (blocks from table_blocks on) the refit: both follow the
-// repack and neither reads what the other writes, so the table build (15 us on its own for 192 patches) runs in the
-// shadow of the refit's chains of dependent loads.
-__global__ void __launch_bounds__(128) k_batch_table_refit(const BatchEntry *__restrict__ entries,
-                                                           const uint32_t *__restrict__ patch_prefix,
-                                                           const uint32_t *__restrict__ greg_prefix, uint32_t n_scenes,
-                                                           uint32_t n_patches, uint32_t n_greg, uint32_t levels,
-                                                           uint32_t refit_blocks)
+__global__ void k_batch_refit(const BatchEntry *__restrict__ entries, const uint32_t *__restrict__ patch_prefix,
+                              uint32_t n_scenes, uint32_t n_patches)
 {
-    if (blockIdx.x >= refit_blocks) {
-        batch_greg_node(entries, greg_prefix, n_scenes, n_greg, levels,
-                        (size_t)(blockIdx.x - refit_blocks) * blockDim.x + threadIdx.x);
-        return;
-    }
-    const uint32_t gp = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gp >= n_patches) return;
-    const uint32_t s = find_scene(patch_prefix, n_scenes, gp);
+    batch_refit_patch(entries, patch_prefix, n_scenes, n_patches, blockIdx.x * blockDim.x + threadIdx.x);
+}
+
+// Block `block` of the build over a batch's scenes that have new points, in the scenes' own update levels: scene s has the
+// blocks from block_prefix[s] on (greg_update_blocks).
+CCS_DEV void batch_greg_block(const BatchEntry *__restrict__ entries, const uint32_t *__restrict__ block_prefix,
+                              uint32_t n_scenes, uint32_t block)
+{
+    const uint32_t s = find_scene(block_prefix, n_scenes, block);
     const BatchEntry &e = entries[s];
-    refit_one(e.nodes, e.leaf_parent, e.leaf_box, e.refit_flags, gp - patch_prefix[s], e.sc.width);
+    if (!e.px) return;
+    const uint32_t D = greg_update_levels(e.tab.n, e.tab.stride), i = (block - block_prefix[s]) * kGregBlock + threadIdx.x;
+    if (i == 0) *e.tab.depth = D;
+    const uint32_t rank = i >> D, m = i & ((1u << D) - 1u);
+    if (rank < e.tab.n && m + 1u < (1u << D)) greg_table_node(e.tab, e.rec, rank, m);
+}
+
+// Gregory box tables of the scenes with new points, and (blocks below refit_blocks) the refit: both follow the
+// repack and neither reads what the other writes, so the table build (15 us on its own for 192 patches) runs in the
+// shadow of the refit's chains of dependent loads.  Every scene has the blocks that its own update needs (update and refit of
+// 1,536 patches, 24 of them Gregory, beside 64,896 Gregory ones: 529 us with the most levels of any scene for all, 74).
+__global__ void __launch_bounds__(kGregBlock) k_batch_table_refit(const BatchEntry *__restrict__ entries,
+                                                                  const uint32_t *__restrict__ patch_prefix,
+                                                                  const uint32_t *__restrict__ block_prefix,
+                                                                  uint32_t n_scenes, uint32_t n_patches,
+                                                                  uint32_t refit_blocks)
+{
+    if (blockIdx.x >= refit_blocks)
+        batch_greg_block(entries, block_prefix, n_scenes, blockIdx.x - refit_blocks);
+    else
+        batch_refit_patch(entries, patch_prefix, n_scenes, n_patches, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 cudaError_t launch_batch_repack(const BatchEntry *entries, const uint32_t *patch_prefix, uint32_t n_scenes,
@@ -85,23 +99,29 @@ cudaError_t launch_batch_refit(const BatchEntry *entries, const uint32_t *patch_
     return cudaGetLastError();
 }
 
-// The stages after a repack: the tables (n_greg > 0), and the refit when flags are given.
+// The stages after a repack: the tables (greg_blocks > 0), and the refit when flags are given.  In one launch while the
+// refit's blocks are few: beyond, it is bound by how many are resident, and 16 warps per SM of the table's registers
+// against 64 of its own cost more than the table's launch (two scenes, the large one's points unchanged: of 66,432 patches
+// in one launch 51, in two 61 us, of 261,120 98 and 74).
 static cudaError_t launch_batch_table_refit(const BatchEntry *entries, const uint32_t *patch_prefix,
-                                            const uint32_t *greg_prefix, uint32_t n_scenes, uint32_t n_patches,
-                                            uint32_t n_greg, uint32_t levels, uint32_t *flags, uint32_t n_flag_words,
-                                            cudaStream_t s)
+                                            const uint32_t *block_prefix, uint32_t n_scenes, uint32_t n_patches,
+                                            uint32_t greg_blocks, uint32_t *flags, uint32_t n_flag_words, cudaStream_t s)
 {
-    if (n_greg == 0)
-        return flags ? launch_batch_refit(entries, patch_prefix, n_scenes, n_patches, flags, n_flag_words, s) : cudaSuccess;
-    if (flags) {
-        cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(uint32_t) * n_flag_words, s);
+    constexpr uint32_t kMostTogether = 1u << 17;   // patches
+    const bool together = greg_blocks != 0 && flags && n_patches <= kMostTogether;
+    if (greg_blocks != 0) {
+        if (together) {
+            const cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(uint32_t) * n_flag_words, s);
+            if (e != cudaSuccess) return e;
+        }
+        const uint32_t refit_blocks = together ? (n_patches + kGregBlock - 1) / kGregBlock : 0;
+        k_batch_table_refit<<<refit_blocks + greg_blocks, kGregBlock, 0, s>>>(entries, patch_prefix, block_prefix, n_scenes,
+                                                                              n_patches, refit_blocks);
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    const uint32_t refit_blocks = flags ? (n_patches + 127) / 128 : 0;
-    const size_t blocks = refit_blocks + (((size_t)n_greg << levels) + 127) / 128;
-    k_batch_table_refit<<<(unsigned)blocks, 128, 0, s>>>(entries, patch_prefix, greg_prefix, n_scenes, n_patches, n_greg, levels,
-                                                         refit_blocks);
-    return cudaGetLastError();
+    return flags && !together ? launch_batch_refit(entries, patch_prefix, n_scenes, n_patches, flags, n_flag_words, s)
+                              : cudaSuccess;
 }
 
 }  // namespace ccs
@@ -116,8 +136,8 @@ struct ccs_batch {
     BatchEntry *h_table = nullptr;        // pinned host copy, uploaded at the start of every run
     BatchEntry *d_table = nullptr;
     uint32_t *d_ray_prefix = nullptr, *d_patch_prefix = nullptr;
-    uint32_t *d_greg_prefix = nullptr;    // Gregory patches of the scenes that have a box table for them
-    uint32_t n_greg = 0, greg_levels = 0; // their number; the most levels that an update builds
+    uint32_t *d_greg_prefix = nullptr;    // blocks that build the scenes' Gregory box tables after an update
+    uint32_t greg_blocks = 0;             // their number
     uint32_t *d_flags = nullptr;          // refit arrival counters of every scene's nodes
     uint32_t *d_work = nullptr;           // [0] queue head, [1] status word
     void *d_pairs = nullptr;              // the pair engine's scratch (CCS_TRACE_PAIRS), made on first use
@@ -227,16 +247,15 @@ ccs_status ccs_batch_create(ccs_batch **out, ccs_scene *const *scenes, uint32_t 
             t.tab = sc->tab;
             rp[s] = r;
             pp[s] = p;
-            gp[s] = b->n_greg;
-            b->n_greg += sc->tab.n;
-            b->greg_levels = std::max(b->greg_levels, greg_update_levels(sc->tab.n, sc->tab.stride));
+            gp[s] = b->greg_blocks;
+            b->greg_blocks += greg_update_blocks(sc->tab.n, sc->tab.stride);
             r += n_rays[s];
             p += sc->n;
             nn += sc->n_nodes;
         }
         rp[n_scenes] = r;
         pp[n_scenes] = p;
-        gp[n_scenes] = b->n_greg;
+        gp[n_scenes] = b->greg_blocks;
         if ((e = cudaMemcpy(b->d_greg_prefix, gp.data(), sizeof(uint32_t) * (n_scenes + 1), cudaMemcpyHostToDevice)) !=
             cudaSuccess)
             break;
@@ -286,7 +305,7 @@ ccs_status ccs_batch_run(ccs_batch *b, uint32_t stages, const ccs_trace_opts *op
     if (update) BCK(launch_batch_repack(b->d_table, b->d_patch_prefix, b->n, b->n_patches, s));
     if (update || refit)
         BCK(launch_batch_table_refit(b->d_table, b->d_patch_prefix, b->d_greg_prefix, b->n, b->n_patches,
-                                     update ? b->n_greg : 0, b->greg_levels, refit ? b->d_flags : nullptr, b->n_nodes, s));
+                                     update ? b->greg_blocks : 0, refit ? b->d_flags : nullptr, b->n_nodes, s));
     if ((stages & CCS_BATCH_INTERSECT) && use_pairs(cfg)) {
         if (!b->d_pairs) BCK(cudaMalloc(&b->d_pairs, pairs_scratch_bytes(b->n_rays ? b->n_rays : 1)));
         BCK(launch_pairs_batch(b->d_table, b->d_ray_prefix, b->n, b->n_rays, cfg, b->d_pairs, b->d_work + 1,

@@ -19,7 +19,7 @@ namespace ccs {
 
 namespace {
 
-__global__ void __launch_bounds__(128) k_greg_table(GregTabStore t, const float4 *__restrict__ rec, uint32_t D)
+__global__ void __launch_bounds__(kGregBlock) k_greg_table(GregTabStore t, const float4 *__restrict__ rec, uint32_t D)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) *t.depth = D;
@@ -34,8 +34,8 @@ cudaError_t launch_greg_table(const GregTabStore &t, const float4 *rec, bool upd
 {
     if (!t.stride) return cudaSuccess;
     const uint32_t D = update ? greg_update_levels(t.n, t.stride) : t.stride;
-    const size_t n = D ? (size_t)t.n << D : 1;   // (no level: the depth word alone)
-    k_greg_table<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(t, rec, D);
+    const uint32_t blocks = update ? greg_update_blocks(t.n, t.stride) : (uint32_t)((((size_t)t.n << D) + kGregBlock - 1) / kGregBlock);
+    k_greg_table<<<blocks, kGregBlock, 0, s>>>(t, rec, D);
     return cudaGetLastError();
 }
 

@@ -1,4 +1,4 @@
-// Device routines of the Gregory box tables (described in table.cu), shared by its kernels and the batch's refit.
+// Device routines of the Gregory box tables (described in table.cu), shared by its kernel and the batch's.
 #pragma once
 
 #include "table_plan.h"
@@ -22,26 +22,6 @@ CCS_DEV void greg_table_node(const GregTabStore &t, const float4 *__restrict__ r
     float4 *nd = t.node + 4 * (((size_t)rank << t.stride) + table_index(level, path));
 #pragma unroll
     for (int k = 0; k < 3; ++k) nd[k] = make_float4(lmin[k], lmax[k], rmin[k], rmax[k]);
-}
-
-// Thread i of the build over a batch's scenes that have new points: 2^levels threads per Gregory patch (the prefix
-// counts the patches of scenes with a table).
-CCS_DEV void batch_greg_node(const BatchEntry *__restrict__ entries, const uint32_t *__restrict__ prefix,
-                             uint32_t n_scenes, uint32_t n, uint32_t levels, size_t i)
-{
-    const uint32_t p = (uint32_t)(i >> levels), m = (uint32_t)i & ((1u << levels) - 1u);
-    if (p >= n) return;
-    uint32_t lo = 0, hi = n_scenes;   // largest s with prefix[s] <= p
-    while (hi - lo > 1) {
-        const uint32_t h = (lo + hi) >> 1;
-        if (__ldg(prefix + h) <= p) lo = h; else hi = h;
-    }
-    const BatchEntry &e = entries[lo];
-    const uint32_t rank = p - prefix[lo], D = greg_update_levels(e.tab.n, e.tab.stride);
-    if (!e.px) return;
-    if (rank == 0 && m == 0) *e.tab.depth = D;
-    if (m + 1u >= (1u << D)) return;
-    greg_table_node(e.tab, e.rec, rank, m);
 }
 
 }  // namespace ccs

@@ -37,4 +37,14 @@ CCS_TABLE_HD uint32_t greg_update_levels(uint32_t n, uint32_t stored)
     return D;
 }
 
+// Blocks of kGregBlock threads that build those levels, one thread per node (one block for the depth word where no level is
+// built, none for a scene without a table).
+constexpr uint32_t kGregBlock = 128;
+inline uint32_t greg_update_blocks(uint32_t n, uint32_t stored)
+{
+    if (n == 0 || stored == 0) return 0;
+    const uint32_t D = greg_update_levels(n, stored);
+    return D ? (uint32_t)((((uint64_t)n << D) + kGregBlock - 1) / kGregBlock) : 1;
+}
+
 }  // namespace ccs

@@ -64,9 +64,12 @@ def test_hits_after_an_update(n, local):
     fresh.close()
 
 
+# (a batch of more than 2^17 patches refits in a launch of its own)
+@pytest.mark.parametrize("large", [37, 75])
 @pytest.mark.parametrize("moves", ["all", "small", "large"])
-def test_batch_of_scenes_of_very_different_size(moves):
-    parts = [gregory_scene(37), sg.make_scene(4, 0.03, 3, 2), gregory_scene(2), gregory_scene(8), sg.make_scene(3, 0.03, 3, 4)]
+def test_batch_of_scenes_of_very_different_size(moves, large):
+    parts = [gregory_scene(large), sg.make_scene(4, 0.03, 3, 2), gregory_scene(2), gregory_scene(8),
+             sg.make_scene(3, 0.03, 3, 4)]
     parts = [q if isinstance(q, tuple) else (q.P, q.types) for q in parts]
     parts[4] = (parts[4][0], np.zeros_like(parts[4][1]))   # without a Gregory patch
     scenes = [ccs.Scene(P, t, local=True) for P, t in parts]

@@ -15,7 +15,7 @@ int main() {
     unsigned n; unsigned long long bytes;
     while (scanf("%u %llu", &n, &bytes) == 2) {
         const unsigned s = ccs::greg_table_levels(n, bytes);
-        printf("%u %u\n", s, ccs::greg_update_levels(n, s));
+        printf("%u %u %u\n", s, ccs::greg_update_levels(n, s), ccs::greg_update_blocks(n, s));
     }
     return 0;
 }
@@ -34,10 +34,12 @@ def test_stored_and_updated_levels(tmp_path):
     text = "\n".join(f"{n} {b}" for n, b in cases) + "\n"
     out = subprocess.run([str(tmp_path / "h")], input=text, capture_output=True, text=True, check=True).stdout.split("\n")
     got = {c: tuple(map(int, q.split())) for c, q in zip(cases, out)}
-    for (n, b), (stored, update) in got.items():
+    for (n, b), (stored, update, blocks) in got.items():
         most = min(b, 1 << 28)
         assert stored <= 16 and (stored == 0 or (n << stored) * 64 <= most), (n, b)
         assert stored == 16 or n == 0 or (n << (stored + 1)) * 64 > most, (n, b)   # as deep as fits
         assert update <= min(stored, 10) and (update == 0 or n << update <= 1 << 16), (n, b)
         assert update == min(stored, 10) or n << (update + 1) > 1 << 16, (n, b)
+        # a scene's blocks cover its own nodes, at least the depth word; a scene without a table has none
+        assert blocks == (0 if stored == 0 else max(1, -(-(n << update) // 128)) if update else 1), (n, b)
     assert [got[(n, BIG)][1] for n in (24, 64, 65, 96, 1536, 4056, 32768, 32769, 64896)] == [10, 10, 9, 9, 5, 4, 1, 0, 0]
