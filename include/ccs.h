@@ -155,7 +155,8 @@ typedef struct {
                                        whose dropped candidates could still hold the answer has its lane
                                        walk the BVH again for the next ones.  Hits are bit-identical.  Uses
                                        about 200 bytes of scratch per ray from a stream-ordered memory
-                                       pool of the library (kept for reuse), on the launch's stream; the
+                                       pool of the library (kept for reuse, ccs_release_scratch), on the
+                                       launch's stream; the
                                        work order, bvh_burst, vote, chunk and min_blocks do not apply, and
                                        blocks_per_sm is what fits.  Counters: slots 8..17 hold candidates
                                        listed, rays that dropped some, walks for dropped candidates,
@@ -220,6 +221,13 @@ ccs_status ccs_scene_create(ccs_scene **out, const float *x, const float *y, con
 ccs_status ccs_scene_update_points(ccs_scene *scene, const float *x, const float *y, const float *z, void *stream);
 
 ccs_status ccs_scene_destroy(ccs_scene *scene);
+
+/* Give the scratch of past launches back: the memory that the library's stream-ordered pool holds on the current device
+ * and that no launch, running or queued, uses.  The pool keeps freed scratch for the next launch, about 200 bytes per ray
+ * of the largest pair-engine launch (CCS_TRACE_PAIRS and launches that leave the engine open) and, over all streams, at
+ * most 4 GB or the largest single launch's scratch where that is more.  The next such launch takes new memory.
+ * Thread-safe; does not synchronise.  Errors: CUDA. */
+ccs_status ccs_release_scratch(void);
 
 /* BVH over whole-patch boxes (AABB of the 16 or 20 control points; convex hull property, Sec. 3.1),
  * built on the host with binned SAH (Sec. 4), one patch per leaf, binary or collapsed to 4-wide nodes

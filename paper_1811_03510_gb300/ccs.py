@@ -137,6 +137,7 @@ _SIGS = {
                               ctypes.c_void_p],
     "ccs_gen_mirror": [ctypes.c_void_p, ctypes.POINTER(ccs_rays), ctypes.POINTER(ccs_hits), ctypes.c_uint32,
                        ctypes.c_uint32, ctypes.c_float, ctypes.POINTER(ccs_rays), ctypes.c_void_p],
+    "ccs_release_scratch": [],
     "ccs_scene_info": [ctypes.c_void_p, ctypes.POINTER(ctypes.c_uint32), ctypes.POINTER(ctypes.c_uint32)],
     "ccs_occluded": [ctypes.c_void_p, ctypes.POINTER(ccs_rays), ctypes.c_uint32, ctypes.c_void_p,
                      ctypes.POINTER(ccs_trace_opts), ctypes.c_void_p],
@@ -546,6 +547,10 @@ def ccs_scene_sync_status(scene: int, stream=None) -> int:
     if st not in (CCS_OK, CCS_ERR_TRAVERSAL_LIMIT):
         _check(st)
     return st
+
+
+def ccs_release_scratch():
+    _check(lib().ccs_release_scratch())
 
 
 def ccs_scene_info(scene: int):

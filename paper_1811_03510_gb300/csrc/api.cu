@@ -417,6 +417,12 @@ ccs_status ccs_scene_destroy(ccs_scene *scene)
     return CCS_OK;
 }
 
+ccs_status ccs_release_scratch(void)
+{
+    CCS_CUDA(pool_trim());
+    return CCS_OK;
+}
+
 ccs_status ccs_scene_info(const ccs_scene *scene, uint32_t *n_patches, uint32_t *n_nodes)
 {
     CCS_ARG(scene, "scene is NULL");

@@ -147,9 +147,10 @@ bool use_pairs(const LaunchCfg &cfg);
 void choose_engine(LaunchCfg &cfg, const ccs_scene *sc, uint32_t n, cudaStream_t s);
 size_t pairs_scratch_bytes(uint32_t n);
 // scratch of one launch from the library's stream-ordered memory pool of the current device (pairs.cu):
-// allocated and freed in the order of `s`; freed memory stays in the pool for reuse
+// allocated and freed in the order of `s`; freed memory stays in the pool for reuse, up to a bound
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);
 cudaError_t pool_free(void *p, cudaStream_t s);
+cudaError_t pool_trim();   // what no launch uses, back to the driver
 cudaError_t launch_pairs_single(const DevScene &sc, const DevRays &r, const DevHits &h, uint32_t n,
                                 const LaunchCfg &cfg, uint32_t *status, int num_sms, cudaStream_t s);
 cudaError_t launch_pairs_batch(const BatchEntry *entries, const uint32_t *ray_prefix, uint32_t n_scenes,

@@ -36,32 +36,47 @@ size_t pairs_scratch_bytes(uint32_t n) { return pair_scratch_bytes(n); }
 
 namespace {
 
-// The library's memory pool of the current device (created on first use; freed memory stays in the pool).
-cudaError_t pair_pool(cudaMemPool_t *out)
+// The library's memory pools, one per device, created on first use.  Freed memory stays in a pool for reuse, as mapping it
+// again would cost a launch more than it takes, up to kPoolKeep, which two of the largest launches that the library gives
+// the pair engine by itself fit in (1.6 GB each), or the largest launch's scratch where that is more; the driver takes the
+// rest back at the next synchronisation, and ccs_release_scratch all that no launch uses.
+constexpr uint64_t kPoolKeep = (uint64_t)4 << 30;
+struct ScratchPool {
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = 0;   // the release threshold set
+};
+std::mutex g_pool_mu;   // of the table
+ScratchPool *current_pool()
 {
     constexpr int kMaxDevices = 64;
-    static cudaMemPool_t pools[kMaxDevices] = {};
-    static std::mutex mu;
+    static ScratchPool pools[kMaxDevices];
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!pools[dev]) {
+    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices ? &pools[dev] : nullptr;
+}
+
+// The pool of the current device for a launch that takes `bytes` of it.
+cudaError_t pool_for(uint64_t bytes, cudaMemPool_t *out)
+{
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    ScratchPool *p = current_pool();
+    if (!p) return cudaErrorInvalidDevice;
+    cudaError_t e;
+    if (!p->pool) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t p = nullptr;
-        if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
-        uint64_t keep = ~0ull;
-        if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
-            cudaMemPoolDestroy(p);
+        if ((e = cudaGetDevice(&props.location.id)) != cudaSuccess) return e;
+        if ((e = cudaMemPoolCreate(&p->pool, &props)) != cudaSuccess) {
+            p->pool = nullptr;
             return e;
         }
-        pools[dev] = p;
     }
-    *out = pools[dev];
+    uint64_t keep = bytes > kPoolKeep ? bytes : kPoolKeep;
+    if (keep > p->keep) {
+        if ((e = cudaMemPoolSetAttribute(p->pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
+        p->keep = keep;
+    }
+    *out = p->pool;
     return cudaSuccess;
 }
 
@@ -93,12 +108,20 @@ cudaError_t cand_pass(const Src &src, const PairBufs &pb, const LaunchCfg &cfg, 
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s)
 {
     cudaMemPool_t pool = nullptr;
-    const cudaError_t e = pair_pool(&pool);
+    const cudaError_t e = pool_for(bytes, &pool);
     if (e != cudaSuccess) return e;
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 
 cudaError_t pool_free(void *p, cudaStream_t s) { return cudaFreeAsync(p, s); }
+
+cudaError_t pool_trim()
+{
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    ScratchPool *p = current_pool();
+    if (!p) return cudaErrorInvalidDevice;
+    return p->pool ? cudaMemPoolTrimTo(p->pool, 0) : cudaSuccess;
+}
 
 cudaError_t launch_pairs_single(const DevScene &sc, const DevRays &r, const DevHits &h, uint32_t n,
                                 const LaunchCfg &cfg, uint32_t *status, int num_sms, cudaStream_t s)
