@@ -205,7 +205,10 @@ typedef struct {
  *   to z, y = z x x (the world axes where that is degenerate).  The BVH and the patch root interval stay
  *   in world space.  The hits are those of the same method with boxes in these frames.
  * The library copies the data into its own device store (patch records anchored at their box centre,
- * Sec. 3.4); the caller keeps ownership of its arrays.  n_patches may be 0 (every ray misses).
+ * Sec. 3.4); the caller keeps ownership of its arrays.  Device memory: 353 bytes per patch, and for Gregory patches a table
+ * of their sub-domain boxes that the pair engine and the learned traversal read: 2^16 boxes of 64 bytes (4.2 MB) per
+ * Gregory patch, halved until the table is at most 256 MB and 1/32 of the free device memory (24 Gregory patches 101 MB,
+ * 64 or more between 128 and 256 MB); where it cannot be had there is none.  n_patches may be 0 (every ray misses).
  * Blocks until the copy has finished.  Errors: INVALID_ARG (null pointers, n_patches > 2^26),
  * OOM, CUDA. */
 ccs_status ccs_scene_create(ccs_scene **out, const float *x, const float *y, const float *z, const uint8_t *types,
