@@ -147,13 +147,40 @@ def whole_job_rate(rays_per_step: int, steps: int, t_slowest: float, world: int)
     return rays_per_step * world * steps / t_slowest / 1e6
 
 
-def engine_of(o) -> str:
+def leaves_engine_open(o) -> bool:
+    """Options that leave the engine to the library (include/ccs.h, ccs_trace_opts.flags)."""
+    return not o.flags and not any(getattr(o, k) for k in ("block_threads", "blocks_per_sm", "chunk", "bvh_burst", "min_blocks",
+                                                           "vote", "iter_cap", "pixel_spread")) and o.lanes_per_ray <= 1
+
+
+def closed_opts(o, n: int, n_patches: int, local: bool):
+    """The options with the engine that the library picks for n rays written out (csrc/engine_plan.h), so that a launch with
+    counters, whose flag closes the choice, runs the kernels that the timed launch runs."""
+    from paper_1811_03510_gb300 import ccs
+    if not leaves_engine_open(o):
+        return o
+    d = ccs.opts_dict(o)
+    if 32 <= n <= 1 << 23 and (local or d["leaf_depth"] == 0 or d["leaf_depth"] > 3 or n > 16 * n_patches):
+        d.update(pairs=True, refill=min(d["refill"] or 8, 24),
+                 cache_slots=1 if d["cache_slots"] == ccs.CCS_CACHE_DEFAULT else d["cache_slots"])
+    else:
+        d.update(chunk=32)
+    return ccs.make_opts(**d)
+
+
+def ray_kernel_opts(o) -> dict:
+    """make_opts arguments of the same options on the ray-persistent kernel (an option of its own asks for it)."""
     from paper_1811_03510_gb300 import ccs
     d = ccs.opts_dict(o)
-    # options that leave the engine open get the pair engine (include/ccs.h, ccs_trace_opts.flags)
-    open_ = not o.flags and not any(d[k] for k in ("block_threads", "blocks_per_sm", "chunk", "bvh_burst", "min_blocks",
-                                                   "vote")) and not o.iter_cap and not o.pixel_spread
-    return "pairs" if (d["pairs"] or open_) and d["lanes_per_ray"] != 3 else ("ray+order" if d["order"] else "ray")
+    d.update(pairs=False, chunk=d["chunk"] or 32)
+    return d
+
+
+def engine_of(o) -> str:
+    """The engine of closed options."""
+    from paper_1811_03510_gb300 import ccs
+    d = ccs.opts_dict(o)
+    return "pairs" if d["pairs"] and d["lanes_per_ray"] != 3 else ("ray+order" if d["order"] else "ray")
 
 
 def kernels_per_launch(o) -> int:
@@ -195,7 +222,7 @@ def kernel_source_hash() -> str:
     import hashlib
     h = hashlib.sha256()
     for f in ("traverse.cuh", "intersect_impl.cuh", "intersect.cu", "intersect4.cu", "order.cu", "order_plan.h",
-              "learned.cuh", "ccs_internal.h", "pairs.cuh", "pairs.cu", "pairs_launch.cuh", "pairs_plain.cu"):
+              "learned.cuh", "ccs_internal.h", "cand_plan.h", "pairs.cuh", "pairs.cu", "pairs_launch.cuh", "pairs_plain.cu"):
         with open(os.path.join(ROOT, "paper_1811_03510_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -469,12 +496,11 @@ def run_shadow(args, dev, stream, flush):
 def run_screen(args, dev, stream, scene, prim, n_prim, flush, opts_p):
     """Primary rays with screen-space termination (Sec. 3.3) at the camera's pixel size, against the fixed
     leaf depth of the benchmark, on the same rays and launch options.  Both arms run the ray-persistent
-    kernel: the pair engine has no screen-space mode, so its flag is cleared for both."""
+    kernel: the pair engine has no screen-space mode, so it is asked for with both."""
     import torch
     from paper_1811_03510_gb300 import ccs
     spread = 2.0 * np.tan(np.radians(30.0)) / args.height   # 60 degree vertical field of view
-    base = ccs.opts_dict(opts_p)
-    base["pairs"] = False
+    base = ray_kernel_opts(opts_p)
     out = {"pixel_spread": spread, "engine": "ray-persistent (both arms)"}
     hits = ccs.alloc_hits(n_prim, dev)
     for name, sp in (("fixed_depth", 0.0), ("screen_space", spread)):
@@ -824,7 +850,8 @@ def main():
     for name, arg in (("primary", args.opts_primary), ("diffuse", args.opts_diffuse)):
         if arg:
             tuned[name] = ccs.make_opts(**{"leaf_depth": 8, **json.loads(arg)})
-    opts_p, opts_d = tuned["primary"], tuned["diffuse"]
+    opts_p = closed_opts(tuned["primary"], n_prim, s.n, scene.local)
+    opts_d = closed_opts(tuned["diffuse"], n_diff, s.n, scene.local)
 
     # algorithmic work per launch from the traversal counters (separate, untimed launches)
     counts = {}
