@@ -1,5 +1,5 @@
 """The first launches of a process, in a process of their own: several threads whose first calls have leaf depths (shared
-memory sizes) of their own."""
+memory sizes) of their own, and a capture whose warm-up was the same call outside of it, which takes another engine."""
 import os
 import subprocess
 import sys
@@ -61,6 +61,36 @@ for k, L in enumerate(DEPTHS):
 print("OK")
 '''
 
+CAPTURE = HEAD + r'''
+hits, occ = ccs.alloc_hits(n), torch.zeros(n, dtype=torch.uint8, device="cuda")
+
+
+def step():
+    ccs.ccs_intersect(sc.handle, rays, n, hits)
+    ccs.ccs_occluded(sc.handle, rays, n, occ)
+
+
+side = torch.cuda.Stream()
+side.wait_stream(torch.cuda.current_stream())
+with torch.cuda.stream(side):   # the warm-up: the pair engine
+    for _ in range(3):
+        step()
+torch.cuda.current_stream().wait_stream(side)
+torch.cuda.synchronize()
+ref = ccs.hits_to_numpy(hits)
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g):       # the ray-persistent kernel, for the first time in this process
+    step()
+for p in hits:
+    p.fill_(-3)
+occ.fill_(7)
+g.replay()
+torch.cuda.synchronize()
+assert same(ccs.hits_to_numpy(hits), ref)
+assert np.array_equal(occ.cpu().numpy().astype(bool), ref["pid"] != 0xFFFFFFFF) and int(occ.max()) == 1
+print("OK")
+'''
+
 
 @pytest.fixture(scope="module", autouse=True)
 def dev():
@@ -77,3 +107,7 @@ def run_alone(code):
 
 def test_first_calls_of_threads_with_their_own_leaf_depths():
     run_alone(THREADS)
+
+
+def test_capture_after_a_warm_up_with_the_same_call():
+    run_alone(CAPTURE)
