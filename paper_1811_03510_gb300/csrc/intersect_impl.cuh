@@ -89,7 +89,9 @@ struct BatchSource {
         local = i - __ldg(ray_prefix + lo);
         lsc.s = lo;
     }
-    CCS_DEV bool world_boxes() const { return entries[0].sc.local == 0; }   // (scenes of a batch are mostly alike)
+    // (by the first scene, as scenes of a batch are mostly alike.  Two scenes of 1,536 patches and 920 k rays of one of them,
+    // the other first or last: rays in world axes 479 / 450 us, in local frames 250 / 262)
+    CCS_DEV bool world_boxes() const { return entries[0].sc.local == 0; }
     CCS_DEV const DevRays &rays_of(uint32_t s) const { return entries[s].rays; }
     CCS_DEV const DevHits &hits_of(uint32_t s) const { return entries[s].hits; }
 };

@@ -23,15 +23,16 @@ constexpr int kOffW1 = 0, kOffB1 = 1536, kOffW2 = 1600, kOffB2 = 5696, kOffW3 = 
 // kTile samples that stay in shared memory with the weights; k_mlp_reduce adds the blocks' shares and, in a training
 // step, applies Adam and publishes the BF16 copy.
 //
-// Bound: 55 k multiply-adds per sample in FP32 (the masters' precision), so FP32 issue and the shared-memory
-// bandwidth that feeds it.  A thread owns a 4 x 4 tile of every product (8 x 4 of the weight gradients, which stay
-// in its registers over all of the block's tiles), fed by 16-byte loads: 2 loads per 16 multiply-adds.  Rows are
-// padded to 28 or 68 floats, so that 8 threads that read 8 rows hit 32 banks.  32 samples per tile give 256 blocks at
-// a batch of 8,192, two per SM; 64 would leave a sixth of the SMs without one.
-// Measured on GB300, batch 8,192: a gradient call 25 us (this kernel 24 us, 19 T FMA/s, and the reduction 5 us, under
-// ncu), before 177 us (one thread per sample with its layers in local memory 95 us, one thread per parameter and
-// 512 samples with atomics 92 us).  Error against 64 bits 1.7e-7, before 1.4e-6; no atomics, so the sums are the same
-// every time.
+// Bound: 27.6 k multiply-adds per sample in FP32 (the masters' precision; forward 9,728, backward 8,192, weight gradients
+// 9,728), so FP32 issue, 5.6 us at a batch of 8,192, and the shared-memory bandwidth that feeds it.  A thread owns a 4 x 4
+// tile of every product (8 x 4 of the weight gradients, which stay in its registers over all of the block's tiles), fed by
+// 16-byte loads: 2 loads per 16 multiply-adds.  Rows are padded to 28 or 68 floats, so that 8 threads that read 8 rows hit
+// 32 banks.  32 samples per tile give 256 blocks at a batch of 8,192, two per SM; 64 would leave a sixth of the SMs without
+// one.
+// Measured on GB300, batch 8,192: a gradient call 25 us (this kernel 24 us, 9.4 T FMA/s or 23% of the lanes' rate, and the
+// reduction 5 us, under ncu), before 177 us (one thread per sample with its layers in local memory 95 us, one thread per
+// parameter and 512 samples with atomics 92 us).  Error against 64 bits 1.7e-7, before 1.4e-6; no atomics, so the sums are
+// the same every time.
 // ------------------------------------------------------------------------------------------------
 constexpr int kTile = 32, kGradThreads = 128;
 constexpr int kXs = 28, kHs = 68;                  // row strides in shared memory (24 and 64 columns)

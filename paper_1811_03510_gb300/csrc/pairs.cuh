@@ -4,7 +4,8 @@
 //     patches, ordered by (entry distance of the patch box, patch id).  Before the list is full nothing
 //     is pruned but [tmin, tmax]; once it is full, subtrees that enter beyond its last entry are skipped
 //     and the smallest entry distance dropped that way is kept (t_evict).  A Bezier patch whose root box in its
-//     own frame the ray does not come near is no candidate (root_box_near: its pair would record no leaf).  A ray with candidates becomes a task with a cost class (the highest when a candidate is a Gregory patch, else its number of
+//     own frame the ray does not come near is no candidate (root_box_near: its pair would record no leaf).  A ray with
+//     candidates becomes a task with a cost class (the highest when a candidate is a Gregory patch, else its number of
 //     candidates); rays with no candidate are written as misses here.
 //  2. Each task's index goes to the list of its cost class (the candidate pass counts the classes' places),
 //     and the subdivision pass's queue takes the classes costliest first, so that the long rays start
@@ -231,17 +232,18 @@ CCS_DEV void list_patch(const DevScene &sc, uint32_t p, float n0, const float (&
 // entered beyond its last entry are skipped and the smallest entry distance dropped that way is kept (t_evict).  Bezier
 // patches whose root box the ray does not come near are no candidates (root_box_near).  Returns false when the
 // iteration budget it ran out.
-template <bool STATS, int BW>
+template <int BW>
 CCS_DEV bool walk_candidates(const DevScene &sc, const RayG<3> &r, const float (&ro)[3], const float (&rd)[3],
                              float tmin, float tmax, float leaf, float lb_t, uint32_t lb_p, uint32_t &it,
                              float (&kt)[kPairCands], uint32_t (&kp)[kPairCands], int &cnt, float &t_evict,
-                             bool &evicted, unsigned long long &nodes, unsigned long long &culled, const Grp &G)
+                             bool &evicted, const Grp &G)
 {
     constexpr int C = kPairCands;
     const float kInf = __int_as_float(0x7f800000);
     int2 stk[kBvhStack];
     int sp = 0, node = 0;
     float n0 = tmin;
+    unsigned long long none = 0;   // (its culls are not counted)
     for (;;) {
         if (node == kDone) break;
         if (it == 0) return false;
@@ -250,9 +252,8 @@ CCS_DEV bool walk_candidates(const DevScene &sc, const RayG<3> &r, const float (
             const uint32_t p = (uint32_t)(~node);
             // (not one that an earlier walk listed)
             if (cand_less(lb_t, lb_p, n0, p))
-                list_patch<STATS>(sc, p, n0, ro, rd, tmin, leaf, kt, kp, cnt, t_evict, evicted, culled, G);
+                list_patch<false>(sc, p, n0, ro, rd, tmin, leaf, kt, kp, cnt, t_evict, evicted, none, G);
         } else {
-            ++nodes;
             // once the list is full, a subtree entered beyond its last entry only holds dropped patches
             const float bound = cnt == C ? kt[C - 1] : tmax;
             if constexpr (BW == 4) {
@@ -726,14 +727,13 @@ __device__ __forceinline__ MoreCands collect_more(const DevScene sc, const float
     out.cnt = 0;
     out.t_evict = __int_as_float(0x7f800000);
     out.evicted = false;
-    unsigned long long nodes = 0, culled = 0;
     Grp G;
     G.c = 0;
     G.mask = 0xffffffffu;
     G.l0 = G.l1 = G.l2 = threadIdx.x & 31;
     uint32_t it = iter_cap;
-    out.capped = !walk_candidates<false, BW>(sc, r, ro, rd, rs[6 * stride], rs[7 * stride], leaf, lb_t, lb_p, it, kt, kp,
-                                             out.cnt, out.t_evict, out.evicted, nodes, culled, G);
+    out.capped = !walk_candidates<BW>(sc, r, ro, rd, rs[6 * stride], rs[7 * stride], leaf, lb_t, lb_p, it, kt, kp, out.cnt,
+                                      out.t_evict, out.evicted, G);
     if (!out.capped)
         for (int j = 0; j < out.cnt; ++j) dst[j] = make_uint2(kp[j], __float_as_uint(kt[j]));
     return out;
