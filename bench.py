@@ -169,9 +169,14 @@ def closed_opts(o, n: int, n_patches: int, local: bool):
 
 
 def ray_kernel_opts(o) -> dict:
-    """make_opts arguments of the same options on the ray-persistent kernel (an option of its own asks for it)."""
+    """make_opts arguments of the same options on the ray-persistent kernel (an option of its own asks for it).  The pair engine
+    has no use for the other kernel's options, so a tuner that chose it leaves them at whatever noise made them: the
+    defaults (a tuned min_blocks of 4 took the kernel from 2136 to 1516 MRays/s)."""
     from paper_1811_03510_gb300 import ccs
     d = ccs.opts_dict(o)
+    if d["pairs"]:
+        d.update(block_threads=0, blocks_per_sm=0, chunk=0, bvh_burst=0, min_blocks=0, vote=0, refill=0,
+                 cache_slots=ccs.CCS_CACHE_DEFAULT)
     d.update(pairs=False, chunk=d["chunk"] or 32)
     return d
 

@@ -29,3 +29,11 @@ def test_screen_space_arms_ask_for_the_ray_kernel(kw):
     for spread in (0.0, 0.001):
         o = ccs.make_opts(**bench.ray_kernel_opts(ccs.make_opts(**kw)), pixel_spread=spread)
         assert not bench.leaves_engine_open(o) and bench.engine_of(o) == "ray" and o.chunk == kw.get("chunk", 32)
+
+
+def test_options_tuned_for_the_pair_engine_do_not_reach_the_ray_kernel():
+    d = bench.ray_kernel_opts(ccs.make_opts(pairs=True, min_blocks=4, vote=12, block_threads=96, cache_slots=0, refill=24,
+                                            bvh_width=4, image_width=1920, leaf_depth=7))
+    assert (d["min_blocks"], d["vote"], d["block_threads"], d["refill"], d["cache_slots"]) == (0, 0, 0, 0, ccs.CCS_CACHE_DEFAULT)
+    assert (d["bvh_width"], d["image_width"], d["leaf_depth"], d["chunk"]) == (4, 1920, 7, 32)
+    assert bench.ray_kernel_opts(ccs.make_opts(min_blocks=4, vote=12, chunk=64))["min_blocks"] == 4   # its own stay
